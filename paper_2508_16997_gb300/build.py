@@ -19,7 +19,8 @@ CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "liblbve.so")
 SOURCES = ["lbve_host.cu", "lbve_kernels.cu", "lbve_noalloc.cu", "lbve_adjoint.cu", "lbve_wall.cu"]
-HEADERS = ["lbve_internal.h", "lbve_step.cuh", "lbve_adjoint.cuh", os.path.join("..", "..", "include", "lbve.h")]
+HEADERS = ["lbve_internal.h", "lbve_step.cuh", "lbve_linear.cuh", "lbve_df32.cuh",
+           "lbve_adjoint.cuh", os.path.join("..", "..", "include", "lbve.h")]
 
 NVCC_FLAGS = ["-gencode", "arch=compute_103a,code=sm_103a", "-O3", "-lineinfo", "-std=c++17",
               "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall", f"-I{os.path.join(ROOT, 'include')}"]

@@ -46,6 +46,24 @@ __device__ __forceinline__ df32 operator*(df32 a, df32 b) {
   e = fmaf(a.lo, b.hi, e);
   return df32(p, e);
 }
+// a float32 factor (the exactly representable literals) has no low part
+__device__ __forceinline__ df32 operator*(float a, df32 b) {
+  const float p = a * b.hi;
+  return df32(p, fmaf(a, b.lo, fmaf(a, b.hi, -p)));
+}
+// Literal factor of an expression in R, exactly representable in float32.
+template <typename R>
+struct Literal {
+  using type = R;
+};
+template <>
+struct Literal<df32> {
+  using type = float;
+};
+template <typename R>
+__device__ __forceinline__ constexpr typename Literal<R>::type lit(double x) {
+  return (typename Literal<R>::type)x;
+}
 __device__ __forceinline__ df32 operator/(df32 a, df32 b) {
   // one correctly rounded reciprocal serves both quotients; the correction
   // takes the first quotient's extra rounding (about 47 bits in all)

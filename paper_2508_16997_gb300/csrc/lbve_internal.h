@@ -79,6 +79,14 @@ enum : int {
   kCoefMupLam,  // mu_p/lambda
   kCoefInvL2,   // 1/L^2 of the FENE models (0 for Oldroyd-B)
   kCoefAfene,   // a = 1/(1 - 2/L^2) of FENE-P
+  // products the step uses; d = 1/3 for the 8-byte precisions, whose diagonal
+  // second-order terms carry the factor 1/3, 1 for float32
+  kCoefN1,      // (1 - 1/tau_s1) d / 3
+  kCoefN2,      // (1 - 1/tau_s2) / 3
+  kCoefHs2,     // (1 - 1/(2 tau_s1)) / 2
+  kCoefWd,      // mu_p / (lambda tau_s1) d
+  kCoefWx,      // mu_p / (lambda tau_s1)
+  kCoefP2,      // (1 - 1/tau_p2) d / 3
   kNumCoef
 };
 
@@ -104,7 +112,7 @@ struct alignas(16) InstDev {
   // Collision coefficients rounded once to float32 (cf), their float64
   // values (cd) and the low parts of the LBVE_DF32 pairs (cl = cd - cf), so
   // that no kernel converts precision per node.
-  float cf[16];
+  float cf[20];
   double* fields;                // [6][stride]  rho, ux, uy, Axx, Axy, Ayy (float64)
   const uint8_t* mask;           // [stride] 1 = solid node, or null (no mask)
   double* wall_rec;              // [wall_cap][kWallRec] final-step wall sums
@@ -112,10 +120,11 @@ struct alignas(16) InstDev {
                                  // columns (inlet rows, then outlet rows), deviations
   const double* inlet;           // [5][ny] u_x, u_y, A_xx, A_xy, A_yy at the inlet
   double inv_Uc;
-  double cd[16];
-  float cl[16];
+  double cd[20];
+  float cl[20];
 };
 static_assert(sizeof(InstDev) % 16 == 0, "descriptor size");
+static_assert(kNumCoef <= 20, "coefficient slots");
 
 // One tile of one instance: {instance, x0, y0, partial slot, masked}.
 // masked: the tile holds a solid node or a node with a solid neighbour along

@@ -32,6 +32,7 @@
 
 #include "lbve_df32.cuh"
 #include "lbve_internal.h"
+#include "lbve_linear.cuh"
 
 #ifndef LBVE_FP32_MIN_BLOCKS
 #define LBVE_FP32_MIN_BLOCKS 7
@@ -110,8 +111,9 @@ __device__ __forceinline__ void cde_moments(const R d[9], CdeM<R>& m) {
 // momentum (and the slowly relaxing conformation moments) accumulate over
 // their relaxation times.  The rest population is taken as b0' minus the
 // other eight, which equals its formula in exact arithmetic and keeps
-// sum_i d_i = b0' up to unbiased rounding.  Float64 keeps the plain formula:
-// its weight bias is ~1e-17, and the float64 step is bound by the FP64 pipe.
+// sum_i d_i = b0' up to unbiased rounding.  Float32 pairs keep the plain
+// formula; float64 scales the coefficients by the weights and adds in fixed
+// point (lattice_populations).
 template <typename R>
 __device__ __forceinline__ R wmul(R v, R w, R wlo) {
   if constexpr (sizeof(R) == 4)
@@ -120,34 +122,52 @@ __device__ __forceinline__ R wmul(R v, R w, R wlo) {
     return w * v;
 }
 
-template <typename R>
+// THIRD = false: without third-order coefficients (the conformation lattices).
+// Float32 then adds the zero terms all the same: without them the compiler
+// would contract the remaining products differently, and the roundings of
+// float32 runs stay what they were.
+template <typename R, bool THIRD = true>
 __device__ __forceinline__ void reconstruct(R b0p, R bx, R by, R bxx, R byy, R bxy, R bxxy,
                                             R bxyy, R out[9]) {
-  const R w0 = R(4.0 / 9.0), w1 = R(1.0 / 9.0), w5 = R(1.0 / 36.0);
-  // low parts of 1/9 and 1/36 below their float32 roundings
-  constexpr float kW1lo = (float)(1.0 / 9.0 - (double)(float)(1.0 / 9.0));
-  constexpr float kW5lo = (float)(1.0 / 36.0 - (double)(float)(1.0 / 36.0));
-  const R w1lo = R(kW1lo), w5lo = R(kW5lo);
-  const R s = bxx + byy;
-  if constexpr (sizeof(R) == 8) out[0] = w0 * (b0p - R(1.5) * s);
-  const R b13 = b0p + R(3.0) * bxx - R(1.5) * byy;
-  const R o13 = R(3.0) * bx - R(4.5) * bxyy;
-  out[1] = wmul<R>(b13 + o13, w1, w1lo);
-  out[3] = wmul<R>(b13 - o13, w1, w1lo);
-  const R b24 = b0p - R(1.5) * bxx + R(3.0) * byy;
-  const R o24 = R(3.0) * by - R(4.5) * bxxy;
-  out[2] = wmul<R>(b24 + o24, w1, w1lo);
-  out[4] = wmul<R>(b24 - o24, w1, w1lo);
-  const R bd = b0p + R(3.0) * s;
-  const R xy9 = R(9.0) * bxy;
-  const R o57 = R(3.0) * (bx + by) + R(9.0) * (bxxy + bxyy);
-  const R o68 = R(3.0) * (by - bx) + R(9.0) * (bxxy - bxyy);
-  out[5] = wmul<R>((bd + xy9) + o57, w5, w5lo);
-  out[7] = wmul<R>((bd + xy9) - o57, w5, w5lo);
-  out[6] = wmul<R>((bd - xy9) + o68, w5, w5lo);
-  out[8] = wmul<R>((bd - xy9) - o68, w5, w5lo);
-  if constexpr (sizeof(R) == 4)
-    out[0] = b0p - (((out[1] + out[3]) + (out[2] + out[4])) + ((out[5] + out[7]) + (out[6] + out[8])));
+  if constexpr (std::is_same<R, double>::value) {
+    const double third = 1.0 / 3.0;
+    lattice_populations<THIRD>(b0p * (1.0 / 9.0), bx * third, by * third, bxx * third, byy * third,
+                               bxy, bxxy, bxyy, out);
+  } else {
+    const R w0 = R(4.0 / 9.0), w1 = R(1.0 / 9.0), w5 = R(1.0 / 36.0);
+    // low parts of 1/9 and 1/36 below their float32 roundings
+    constexpr float kW1lo = (float)(1.0 / 9.0 - (double)(float)(1.0 / 9.0));
+    constexpr float kW5lo = (float)(1.0 / 36.0 - (double)(float)(1.0 / 36.0));
+    const R w1lo = R(kW1lo), w5lo = R(kW5lo);
+    const R s = bxx + byy;
+    if constexpr (sizeof(R) == 8) out[0] = w0 * (b0p - lit<R>(1.5) * s);
+    const R b13 = b0p + lit<R>(3.0) * bxx - lit<R>(1.5) * byy;
+    R o13, o24, o57, o68;
+    if constexpr (THIRD || sizeof(R) == 4) {
+      o13 = lit<R>(3.0) * bx - lit<R>(4.5) * bxyy;
+      o24 = lit<R>(3.0) * by - lit<R>(4.5) * bxxy;
+      o57 = lit<R>(3.0) * (bx + by) + lit<R>(9.0) * (bxxy + bxyy);
+      o68 = lit<R>(3.0) * (by - bx) + lit<R>(9.0) * (bxxy - bxyy);
+    } else {
+      o13 = lit<R>(3.0) * bx;
+      o24 = lit<R>(3.0) * by;
+      o57 = lit<R>(3.0) * (bx + by);
+      o68 = lit<R>(3.0) * (by - bx);
+    }
+    out[1] = wmul<R>(b13 + o13, w1, w1lo);
+    out[3] = wmul<R>(b13 - o13, w1, w1lo);
+    const R b24 = b0p - lit<R>(1.5) * bxx + lit<R>(3.0) * byy;
+    out[2] = wmul<R>(b24 + o24, w1, w1lo);
+    out[4] = wmul<R>(b24 - o24, w1, w1lo);
+    const R bd = b0p + lit<R>(3.0) * s;
+    const R xy9 = lit<R>(9.0) * bxy;
+    out[5] = wmul<R>((bd + xy9) + o57, w5, w5lo);
+    out[7] = wmul<R>((bd + xy9) - o57, w5, w5lo);
+    out[6] = wmul<R>((bd - xy9) + o68, w5, w5lo);
+    out[8] = wmul<R>((bd - xy9) - o68, w5, w5lo);
+    if constexpr (sizeof(R) == 4)
+      out[0] = b0p - (((out[1] + out[3]) + (out[2] + out[4])) + ((out[5] + out[7]) + (out[6] + out[8])));
+  }
 }
 
 // Pull the nine populations of one lattice arriving at (x, y): d_i(x) =
@@ -299,29 +319,6 @@ __device__ __forceinline__ void neighbour_rows(int y, int nx, int ny, bool py, i
   }
 }
 
-// rho, u of node (gx, gy) at the current time: pull (or equilibrium at
-// init), hydro wall completion, moments (eq_ev_f0).
-template <typename R, int MODE>
-__device__ __forceinline__ void node_rho_u(const void* src, const R* __restrict__ force,
-                                           bool ffield, R Fx0, R Fy0, int S, int nx, int ny,
-                                           bool py, int gx, int gy, R& rho, R& ux, R& uy) {
-  const int k = gy * nx + gx;
-  int rm, rp;
-  neighbour_rows(gy, nx, ny, py, rm, rp);
-  const int xm = gx == 0 ? nx - 1 : gx - 1, xp = gx == nx - 1 ? 0 : gx + 1;
-  const R Fx = ffield ? force[k] : Fx0;
-  const R Fy = ffield ? force[S + k] : Fy0;
-  R d[9];
-  PopSource<R, MODE>::hydro(src, S, nx, k, gy * nx, rm, rp, gx, xm, xp, d);
-  if (MODE == kModeStep && !py && (gy == 0 || gy == ny - 1)) zou_he<R>(d, Fx, Fy, gy == 0);
-  HydroM<R> m;
-  hydro_moments<R>(d, m);
-  rho = R(1) + m.drho;
-  const R irho = R(1) / rho;
-  ux = (m.jx + R(0.5) * Fx) * irho;
-  uy = (m.jy + R(0.5) * Fy) * irho;
-}
-
 template <typename R>
 __device__ __forceinline__ R coef(const InstDev& D, int i);
 template <>
@@ -413,78 +410,476 @@ __device__ __forceinline__ void polymer_terms(const InstDev& D, R d0, R d1, R d2
   }
 }
 
-// Component l (xx, xy, yy) of the source Phi_ab of the conformation
-// equation (Sec. 3.2) with G** = d_g u_b.
-template <typename R>
-__device__ __forceinline__ R source_component(int l, R Axx, R Axy, R Ayy, R Fxx, R Fxy, R Fyy,
-                                              R il, R G00, R G01, R G10, R G11) {
-  const R div = G00 + G11;
-  if (l == 0) return -Fxx * il + R(2) * (Axx * G00 + Axy * G10) + Axx * div;
-  if (l == 1) return -Fxy * il + (Axx * G01 + Axy * G11) + (Axy * G00 + Ayy * G10) + Axy * div;
-  return -Fyy * il + R(2) * (Axy * G01 + Ayy * G11) + Ayy * div;
+// a b + c with one rounding.  Written out in the float64 path, where a result
+// must not depend on which product the compiler would contract (the CTA
+// sizes and the one-lattice-per-warp kernel agree bit for bit).
+__device__ __forceinline__ double mad(double a, double b, double c) { return fma(a, b, c); }
+
+// 1 / v by one step of the cubically convergent iteration x (1 + e + e^2),
+// e = 1 - v x (Householder's method), from the float32 approximate
+// reciprocal: three float64 instructions where the division takes about nine,
+// error below 2^-52 of the result.  Outside [2^-100, 2^100] (and for NaN) it
+// divides.
+__device__ __forceinline__ double recip(double v) {
+  const int hi = __double2hiint(v), lo = __double2loint(v);
+  const unsigned e = ((unsigned)hi >> 20) & 0x7ffu;
+  if (e - 923u > 200u) return 1.0 / v;
+  // v rounded toward zero to float32, and its reciprocal back, by bit patterns
+  const unsigned f = __funnelshift_l((unsigned)lo, (unsigned)(hi & 0x7fffffff) - (896u << 20), 3) |
+                     ((unsigned)hi & 0x80000000u);
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__uint_as_float(f)));
+  const unsigned b = __float_as_uint(r);
+  const double x = __hiloint2double(
+      (int)((((b & 0x7fffffffu) >> 3) + (896u << 20)) | (b & 0x80000000u)), (int)(b << 29));
+  const double t = fma(-v, x, 1.0);
+  return fma(x, fma(t, t, t), x);
 }
 
-// Hydrodynamic TRT-RLB collision of one node (eq_ev_f, eq4, eq5, eq6, F_i)
-// and the store of its 9 post-collision populations.
+// Arithmetic of one node per storage precision: its moments, the differences
+// of its neighbours' values, its source and its collisions up to the Hermite
+// coefficients.  The general form (float32, float32 pairs) follows the paper's
+// formulas; the float64 one below counts float64 instructions.
+template <typename R>
+struct Flow {  // rho, u of one node (eq_ev_f0)
+  R rho, ux, uy;
+  __device__ __forceinline__ void set(const HydroM<R>& m, R Fx, R Fy) {
+    rho = R(1) + m.drho;
+    const R irho = R(1) / rho;
+    ux = (m.jx + lit<R>(0.5) * Fx) * irho;
+    uy = (m.jy + lit<R>(0.5) * Fy) * irho;
+  }
+  __device__ __forceinline__ void pull(const R d[9], R Fx, R Fy) {
+    HydroM<R> m;
+    hydro_moments<R>(d, m);
+    set(m, Fx, Fy);
+  }
+  __device__ __forceinline__ void rest() {
+    rho = R(1);
+    ux = uy = R(0);
+  }
+};
+
+// The halo region of a tile in shared memory.
+template <typename R, int N>
+struct Region {
+  R rho[N], ux[N], uy[N];
+  __device__ __forceinline__ void put(int r, const Flow<R>& f) {
+    rho[r] = f.rho;
+    ux[r] = f.ux;
+    uy[r] = f.uy;
+  }
+};
+
+// G** = d_g u_b (G01 = dx uy), dP: d_x (rho ux^3), d_y (rho uy^3), dR: grad rho
+// (eq_p_G form only).
+template <typename R>
+struct Grad {
+  R G00, G01, G10, G11, dPx, dPy, dRx, dRy;
+};
+
+template <typename R>
+struct Arith {
+  using Hydro = HydroM<R>;
+  using Cde = CdeM<R>;
+  static __device__ __forceinline__ void moments(const R d[9], Hydro& m) { hydro_moments<R>(d, m); }
+  static __device__ __forceinline__ void moments(const R d[9], Cde& m) { cde_moments<R>(d, m); }
+
+  // Second-order differences at region slot ri (central inside, one-sided in
+  // y on wall rows: rows y-2..y+2, only those a wall row needs are read).
+  template <int N>
+  static __device__ __forceinline__ void gradients(const Region<R, N>& Q, int ri, int RW, bool wb,
+                                                   bool wt, const Flow<R>& f, bool density,
+                                                   Grad<R>& G) {
+    const auto half = lit<R>(0.5);
+    G.G00 = half * (Q.ux[ri + 1] - Q.ux[ri - 1]);
+    G.G01 = half * (Q.uy[ri + 1] - Q.uy[ri - 1]);
+    const R cxp = Q.rho[ri + 1] * Q.ux[ri + 1] * Q.ux[ri + 1] * Q.ux[ri + 1];
+    const R cxm = Q.rho[ri - 1] * Q.ux[ri - 1] * Q.ux[ri - 1] * Q.ux[ri - 1];
+    G.dPx = half * (cxp - cxm);
+    G.dRx = density ? half * (Q.rho[ri + 1] - Q.rho[ri - 1]) : R(0);
+    const int a = wb ? ri : (wt ? ri - 2 * RW : ri), b = wb ? ri : (wt ? ri - RW : ri - RW);
+    const int c = wb ? ri + RW : (wt ? ri : ri + RW), e = wb ? ri + 2 * RW : ri;
+    const R r0 = f.rho, ux0 = f.ux, uy0 = f.uy;
+    const R rm2 = Q.rho[a], uxm2 = Q.ux[a], uym2 = Q.uy[a];
+    const R rm1 = Q.rho[b], uxm1 = Q.ux[b], uym1 = Q.uy[b];
+    const R rp1 = Q.rho[c], uxp1 = Q.ux[c], uyp1 = Q.uy[c];
+    const R rp2 = Q.rho[e], uxp2 = Q.ux[e], uyp2 = Q.uy[e];
+    G.dRy = R(0);
+    if (wb) {
+      G.G10 = half * (lit<R>(-3) * ux0 + lit<R>(4) * uxp1 - uxp2);
+      G.G11 = half * (lit<R>(-3) * uy0 + lit<R>(4) * uyp1 - uyp2);
+      G.dPy = half * (lit<R>(-3) * (r0 * uy0 * uy0 * uy0) + lit<R>(4) * (rp1 * uyp1 * uyp1 * uyp1) -
+                      rp2 * uyp2 * uyp2 * uyp2);
+      if (density) G.dRy = half * (lit<R>(-3) * r0 + lit<R>(4) * rp1 - rp2);
+    } else if (wt) {
+      G.G10 = half * (lit<R>(3) * ux0 - lit<R>(4) * uxm1 + uxm2);
+      G.G11 = half * (lit<R>(3) * uy0 - lit<R>(4) * uym1 + uym2);
+      G.dPy = half * (lit<R>(3) * (r0 * uy0 * uy0 * uy0) - lit<R>(4) * (rm1 * uym1 * uym1 * uym1) +
+                      rm2 * uym2 * uym2 * uym2);
+      if (density) G.dRy = half * (lit<R>(3) * r0 - lit<R>(4) * rm1 + rm2);
+    } else {
+      G.G10 = half * (uxp1 - uxm1);
+      G.G11 = half * (uyp1 - uym1);
+      G.dPy = half * (rp1 * uyp1 * uyp1 * uyp1 - rm1 * uym1 * uym1 * uym1);
+      if (density) G.dRy = half * (rp1 - rm1);
+    }
+  }
+
+  // Zero differences along an axis (0: x, 1: y) between two solid nodes.
+  static __device__ __forceinline__ void blocked(int axis, Grad<R>& G) {
+    if (axis == 0) G.G00 = G.G01 = G.dPx = G.dRx = R(0);
+    else G.G10 = G.G11 = G.dPy = G.dRy = R(0);
+  }
+
+  // One-sided differences along one axis next to the solid mask (same rule as
+  // the central and wall-row differences: second order on the fluid side when
+  // two fluid nodes lie there, else first order):
+  //   t:     +1 toward +axis, -1 toward -axis (the fluid side)
+  //   f:     the node; i1: region slot of its fluid neighbour at +t
+  //   has2:  whether the node at +2t is fluid; w: its values
+  template <int N>
+  static __device__ __forceinline__ void one_sided(int axis, int t, const Region<R, N>& Q, int ri,
+                                                   int i1, const Flow<R>& f, bool has2,
+                                                   const Flow<R>& w, Grad<R>& G) {
+    const R r0 = f.rho, ux0 = f.ux, uy0 = f.uy;
+    const R r1 = Q.rho[i1], ux1 = Q.ux[i1], uy1 = Q.uy[i1];
+    const R r2 = w.rho, u2x = w.ux, u2y = w.uy;
+    const R v0 = axis == 0 ? ux0 : uy0, v1 = axis == 0 ? ux1 : uy1, v2 = axis == 0 ? u2x : u2y;
+    const R c0 = r0 * v0 * v0 * v0, c1 = r1 * v1 * v1 * v1, c2 = r2 * v2 * v2 * v2;
+    const R ts = (R)t;
+    R dux, duy, dcube, drho;
+    if (has2) {
+      const R h = lit<R>(0.5) * ts;
+      dux = h * (lit<R>(-3) * ux0 + lit<R>(4) * ux1 - u2x);
+      duy = h * (lit<R>(-3) * uy0 + lit<R>(4) * uy1 - u2y);
+      dcube = h * (lit<R>(-3) * c0 + lit<R>(4) * c1 - c2);
+      drho = h * (lit<R>(-3) * r0 + lit<R>(4) * r1 - r2);
+    } else {
+      dux = ts * (ux1 - ux0);
+      duy = ts * (uy1 - uy0);
+      dcube = ts * (c1 - c0);
+      drho = ts * (r1 - r0);
+    }
+    if (axis == 0) {
+      G.G00 = dux;
+      G.G01 = duy;
+      G.dPx = dcube;
+      G.dRx = drho;
+    } else {
+      G.G10 = dux;
+      G.G11 = duy;
+      G.dPy = dcube;
+      G.dRy = drho;
+    }
+  }
+
+  // Component l (xx, xy, yy) of the source Phi_ab of the conformation
+  // equation (Sec. 3.2).
+  static __device__ __forceinline__ R source(int l, const InstDev& D, R Axx, R Axy, R Ayy, R Fxx,
+                                             R Fxy, R Fyy, const Grad<R>& G) {
+    const R il = coef<R>(D, kCoefInvLam);
+    const R G00 = G.G00, G01 = G.G01, G10 = G.G10, G11 = G.G11;
+    const R div = G00 + G11;
+    if (l == 0) return -Fxx * il + lit<R>(2) * (Axx * G00 + Axy * G10) + Axx * div;
+    if (l == 1) return -Fxy * il + (Axx * G01 + Axy * G11) + (Axy * G00 + Ayy * G10) + Axy * div;
+    return -Fyy * il + lit<R>(2) * (Axy * G01 + Ayy * G11) + Ayy * div;
+  }
+
+  // Hydrodynamic TRT-RLB collision (eq_ev_f, eq4, eq5, eq6, F_i): the Hermite
+  // coefficients b0' (minus the rest value), b_x, b_y, b_xx, b_yy, b_xy,
+  // b_xxy, b_xyy of the post-collision populations.
+  static __device__ __forceinline__ void hydro_coefs(const InstDev& D, const Hydro& hm,
+                                                     const Flow<R>& f, const Grad<R>& G, R Fxx,
+                                                     R Fxy, R Fyy, R Fx, R Fy, R b[8]) {
+    const R rho = f.rho, ux = f.ux, uy = f.uy;
+    const R mpl = coef<R>(D, kCoefMupLam);
+    const R txx = mpl * Fxx, txy = mpl * Fxy, tyy = mpl * Fyy;  // polymer stress (eq_kramer)
+    const R cs2 = R(1.0 / 3.0);
+    const R c1 = coef<R>(D, kCoefCs1), c2 = coef<R>(D, kCoefCs2);
+    const R h1 = coef<R>(D, kCoefHs1), w1 = coef<R>(D, kCoefWs1);
+    const R ruxx = rho * ux * ux, ruyy = rho * uy * uy, ruxy = rho * ux * uy;
+    const R ruxxy = ruxx * uy, ruxyy = ruxy * uy;
+    const R nxx = hm.pxx - cs2 * hm.drho - ruxx;   // A_xx^neq
+    const R nyy = hm.pyy - cs2 * hm.drho - ruyy;   // A_yy^neq
+    const R nxy = hm.pxy - ruxy;                   // A_xy^neq
+    const R nxxy = hm.qxxy - cs2 * hm.jy - ruxxy;  // A_xxy^neq
+    const R nxyy = hm.qxyy - cs2 * hm.jx - ruxyy;  // A_xyy^neq
+    b[0] = hm.drho;
+    b[1] = hm.jx + Fx;  // rho u + (1-1/tau)A_a + F-term
+    b[2] = hm.jy + Fy;
+    b[3] = ruxx + c1 * nxx - h1 * G.dPx - w1 * txx;
+    b[4] = ruyy + c1 * nyy - h1 * G.dPy - w1 * tyy;
+    b[5] = ruxy + c1 * nxy - w1 * txy;
+    b[6] = ruxxy + c2 * nxxy;
+    b[7] = ruxyy + c2 * nxyy;
+  }
+
+  // Conformation TRT-RLB collision of lattice l (eq_g0 with G~_i, F~_i and its
+  // backward time difference): c0' (minus the rest value), c_x, c_y, c_xx, c_yy,
+  // c_xy.  sl, so: the source now and one step back.
+  template <bool MASKED>
+  static __device__ __forceinline__ void cde_coefs(const InstDev& D, int l, const Cde& m,
+                                                   const Flow<R>& f, R sl, R so, R uxo, R uyo,
+                                                   R Fx, R Fy, const Grad<R>& G, R c[6]) {
+    const R rho = f.rho, ux = f.ux, uy = f.uy;
+    const R cs2 = R(1.0 / 3.0);
+    const R ep = coef<R>(D, kCoefEp1), c2 = coef<R>(D, kCoefCp2), h1 = coef<R>(D, kCoefHp1);
+    const R irho = R(1) / rho;
+    const R uxx = ux * ux, uyy = uy * uy, uxy = ux * uy;
+    // the force G~_i sees: F (eq_p_G_1) or F - c_s^2 grad rho (eq_p_G)
+    const bool gt = MASKED && D.gtilde;
+    const R Gx = gt ? Fx - cs2 * G.dRx : Fx, Gy = gt ? Fy - cs2 * G.dRy : Fy;
+    const R phi = (l == 1 ? R(0) : R(1)) + m.dphi;
+    const R Bx = m.jx - phi * ux, By = m.jy - phi * uy;
+    const R Bxx = m.pxx - cs2 * m.dphi - phi * uxx;
+    const R Byy = m.pyy - cs2 * m.dphi - phi * uyy;
+    const R Bxy = m.pxy - phi * uxy;
+    // small source terms first, one rounding at the magnitude of phi
+    c[0] = m.dphi + (lit<R>(1.5) * sl - lit<R>(0.5) * so);
+    const R pr = phi * irho;
+    // (1 - 1/tau_p1) B = -B + ep B, kept split so float32 keeps the tiny
+    // difference tau_p1 - 1/2 accurately
+    c[1] = (phi * ux - Bx) + ep * Bx + h1 * (pr * Gx + ux * sl) +
+           lit<R>(0.5) * h1 * (ux * sl - uxo * so);
+    c[2] = (phi * uy - By) + ep * By + h1 * (pr * Gy + uy * sl) +
+           lit<R>(0.5) * h1 * (uy * sl - uyo * so);
+    c[3] = phi * uxx + c2 * Bxx;
+    c[4] = phi * uyy + c2 * Byy;
+    c[5] = phi * uxy + c2 * Bxy;
+  }
+
+  static __device__ __forceinline__ void hydro_populations(const R b[8], R out[9]) {
+    reconstruct<R>(b[0], b[1], b[2], b[3], b[4], b[5], b[6], b[7], out);
+  }
+  static __device__ __forceinline__ void cde_populations(const R c[6], R out[9]) {
+    reconstruct<R, false>(c[0], c[1], c[2], c[3], c[4], c[5], R(0), R(0), out);
+  }
+};
+
+// ---- float64: 162 float64 instructions per node beside the fixed-point sums ------
+// The same formulas with fewer float64 instructions: rho u is j + F/2;
+// second-order terms off c_s^2 come from the sums as three times their value;
+// differences and cubes are shared (cubes in the region instead of the
+// density, differences as twice their value); the diagonal second-order
+// terms carry the weight 1/3 with which lattice_populations takes them
+// (folded into the coefficients kCoefN1, kCoefWd, kCoefP2).
+template <>
+struct Flow<double> {
+  double rho, irho, hx, hy, ux, uy;  // (hx, hy) = rho u
+  template <typename M>
+  __device__ __forceinline__ void set(const M& m, double Fx, double Fy) {
+    rho = 1.0 + m.drho;
+    irho = recip(rho);
+    hx = mad(0.5, Fx, m.jx);
+    hy = mad(0.5, Fy, m.jy);
+    ux = hx * irho;
+    uy = hy * irho;
+  }
+  __device__ __forceinline__ void pull(const double d[9], double Fx, double Fy) {
+    Moments<double> m;
+    lattice_moments<false>(d, m);
+    set(m, Fx, Fy);
+  }
+  // rho u_x^3 / 3, rho u_y^3 / 3
+  __device__ __forceinline__ double cube_x() const { return hx * (1.0 / 3.0) * ux * ux; }
+  __device__ __forceinline__ double cube_y() const { return hy * (1.0 / 3.0) * uy * uy; }
+  __device__ __forceinline__ void rest() {
+    rho = irho = 1.0;
+    hx = hy = ux = uy = 0.0;
+  }
+};
+
+template <int N>
+struct Region<double, N> {
+  double rho[N], ux[N], uy[N], cx[N], cy[N];  // rho: read in the eq_p_G form only
+  __device__ __forceinline__ void put(int r, const Flow<double>& f) {
+    rho[r] = f.rho;
+    ux[r] = f.ux;
+    uy[r] = f.uy;
+    cx[r] = f.cube_x();
+    cy[r] = f.cube_y();
+  }
+};
+
+// All twice the differences; the cubes' in units of Flow::cube_x.
+template <>
+struct Grad<double> {
+  double D00, D01, D10, D11, dcx, dcy, dRx, dRy;
+};
+
+template <>
+struct Arith<double> {
+  struct Hydro {
+    double drho, jx, jy, nxx, nyy, pxy, nxxy, nxyy;
+  };
+  struct Cde {
+    double dphi, jx, jy, nxx, nyy, pxy;
+  };
+  static __device__ __forceinline__ void moments(const double d[9], Hydro& m) {
+    Moments<double> s;
+    lattice_moments<true>(d, s);
+    m = Hydro{s.drho, s.jx, s.jy, s.nxx, s.nyy, s.pxy, s.nxxy, s.nxyy};
+  }
+  static __device__ __forceinline__ void moments(const double d[9], Cde& m) {
+    Moments<double> s;
+    lattice_moments<false>(d, s);
+    m = Cde{s.drho, s.jx, s.jy, s.nxx, s.nyy, s.pxy};
+  }
+
+  // Twice the one-sided difference of a quantity from its value and those one
+  // and two nodes inward, for an inward direction of +1.
+  static __device__ __forceinline__ double inward(double q0, double q1, double q2) {
+    return mad(4.0, q1, mad(-3.0, q0, -q2));
+  }
+  static __device__ __forceinline__ double along_y(const double* q, int ri, int RW, bool wb,
+                                                   bool wt) {
+    if (wb) return inward(q[ri], q[ri + RW], q[ri + 2 * RW]);
+    if (wt) return -inward(q[ri], q[ri - RW], q[ri - 2 * RW]);
+    return q[ri + RW] - q[ri - RW];
+  }
+  template <int N>
+  static __device__ __forceinline__ void gradients(const Region<double, N>& Q, int ri, int RW,
+                                                   bool wb, bool wt, const Flow<double>& f,
+                                                   bool density, Grad<double>& G) {
+    G.D00 = Q.ux[ri + 1] - Q.ux[ri - 1];
+    G.D01 = Q.uy[ri + 1] - Q.uy[ri - 1];
+    G.D10 = along_y(Q.ux, ri, RW, wb, wt);
+    G.D11 = along_y(Q.uy, ri, RW, wb, wt);
+    G.dcx = Q.cx[ri + 1] - Q.cx[ri - 1];
+    G.dcy = along_y(Q.cy, ri, RW, wb, wt);
+    G.dRx = density ? Q.rho[ri + 1] - Q.rho[ri - 1] : 0.0;
+    G.dRy = density ? along_y(Q.rho, ri, RW, wb, wt) : 0.0;
+  }
+  static __device__ __forceinline__ void blocked(int axis, Grad<double>& G) {
+    if (axis == 0) G.D00 = G.D01 = G.dcx = G.dRx = 0.0;
+    else G.D10 = G.D11 = G.dcy = G.dRy = 0.0;
+  }
+  static __device__ __forceinline__ double side(int t, double q0, double q1, bool has2, double q2) {
+    const double ts = (double)t;
+    return has2 ? ts * inward(q0, q1, q2) : 2.0 * ts * (q1 - q0);
+  }
+  template <int N>
+  static __device__ __forceinline__ void one_sided(int axis, int t, const Region<double, N>& Q,
+                                                   int ri, int i1, const Flow<double>& f,
+                                                   bool has2, const Flow<double>& w,
+                                                   Grad<double>& G) {
+    const double dux = side(t, f.ux, Q.ux[i1], has2, w.ux);
+    const double duy = side(t, f.uy, Q.uy[i1], has2, w.uy);
+    const double drho = side(t, f.rho, Q.rho[i1], has2, w.rho);
+    if (axis == 0) {
+      G.D00 = dux;
+      G.D01 = duy;
+      G.dcx = side(t, Q.cx[ri], Q.cx[i1], has2, w.cube_x());
+      G.dRx = drho;
+    } else {
+      G.D10 = dux;
+      G.D11 = duy;
+      G.dcy = side(t, Q.cy[ri], Q.cy[i1], has2, w.cube_y());
+      G.dRy = drho;
+    }
+  }
+
+  static __device__ __forceinline__ double source(int l, const InstDev& D, double Axx, double Axy,
+                                                  double Ayy, double Fxx, double Fxy, double Fyy,
+                                                  const Grad<double>& G) {
+    const double il = D.cd[kCoefInvLam], div2 = G.D00 + G.D11;
+    if (l == 0) return mad(-il, Fxx, mad(Axx, mad(0.5, div2, G.D00), Axy * G.D10));
+    if (l == 2) return mad(-il, Fyy, mad(Ayy, mad(0.5, div2, G.D11), Axy * G.D01));
+    return mad(-il, Fxy, mad(0.5, mad(Axx, G.D01, Ayy * G.D10), Axy * div2));
+  }
+
+  // b_xx and b_yy come divided by 3.
+  static __device__ __forceinline__ void hydro_coefs(const InstDev& D, const Hydro& m,
+                                                     const Flow<double>& f, const Grad<double>& G,
+                                                     double Fxx, double Fxy, double Fyy, double Fx,
+                                                     double Fy, double b[8]) {
+    const double kn = D.cd[kCoefN1], kh = D.cd[kCoefHs2], kw = D.cd[kCoefWd], kt = D.cd[kCoefN2];
+    const double rxx = f.hx * (1.0 / 3.0) * f.ux, ryy = f.hy * (1.0 / 3.0) * f.uy;
+    const double rxy = f.hx * f.uy, rxxy = rxy * f.ux, rxyy = rxy * f.uy;
+    b[0] = m.drho;
+    b[1] = m.jx + Fx;
+    b[2] = m.jy + Fy;
+    b[3] = mad(-kw, Fxx, mad(-kh, G.dcx, mad(kn, mad(-9.0, rxx, m.nxx), rxx)));
+    b[4] = mad(-kw, Fyy, mad(-kh, G.dcy, mad(kn, mad(-9.0, ryy, m.nyy), ryy)));
+    b[5] = mad(-D.cd[kCoefWx], Fxy, mad(D.cd[kCoefCs1], m.pxy - rxy, rxy));
+    b[6] = mad(kt, mad(-3.0, rxxy, m.nxxy), rxxy);
+    b[7] = mad(kt, mad(-3.0, rxyy, m.nxyy), rxyy);
+  }
+
+  // c_xx and c_yy come divided by 3.
+  template <bool MASKED>
+  static __device__ __forceinline__ void cde_coefs(const InstDev& D, int l, const Cde& m,
+                                                   const Flow<double>& f, double sl, double so,
+                                                   double uxo, double uyo, double Fx, double Fy,
+                                                   const Grad<double>& G, double c[6]) {
+    const double ep = D.cd[kCoefEp1], h1 = D.cd[kCoefHp1], kn = D.cd[kCoefP2];
+    const double ux = f.ux, uy = f.uy;
+    const bool gt = MASKED && D.gtilde;
+    const double Gx = gt ? mad(-1.0 / 6.0, G.dRx, Fx) : Fx;
+    const double Gy = gt ? mad(-1.0 / 6.0, G.dRy, Fy) : Fy;
+    const double phi = l == 1 ? m.dphi : 1.0 + m.dphi;
+    const double Bx = mad(-phi, ux, m.jx), By = mad(-phi, uy, m.jy);
+    const double s15 = 1.5 * sl, s05 = 0.5 * so;
+    c[0] = m.dphi + (s15 - s05);
+    const double pr = phi * f.irho;
+    c[1] = mad(h1, mad(pr, Gx, mad(ux, s15, -(uxo * s05))), mad(ep, Bx, mad(phi, ux, -Bx)));
+    c[2] = mad(h1, mad(pr, Gy, mad(uy, s15, -(uyo * s05))), mad(ep, By, mad(phi, uy, -By)));
+    const double ph = phi * (1.0 / 3.0);
+    const double pxx = ph * (ux * ux), pyy = ph * (uy * uy), pxy = phi * (ux * uy);
+    c[3] = mad(kn, mad(-9.0, pxx, m.nxx), pxx);
+    c[4] = mad(kn, mad(-9.0, pyy, m.nyy), pyy);
+    c[5] = mad(D.cd[kCoefCp2], m.pxy - pxy, pxy);
+  }
+
+  static __device__ __forceinline__ void hydro_populations(const double b[8], double out[9]) {
+    lattice_populations<true>(b[0] * (1.0 / 9.0), b[1] * (1.0 / 3.0), b[2] * (1.0 / 3.0), b[3],
+                              b[4], b[5], b[6], b[7], out);
+  }
+  static __device__ __forceinline__ void cde_populations(const double c[6], double out[9]) {
+    lattice_populations<false>(c[0] * (1.0 / 9.0), c[1] * (1.0 / 3.0), c[2] * (1.0 / 3.0), c[3],
+                               c[4], c[5], 0.0, 0.0, out);
+  }
+};
+
+// Flow of node (gx, gy) at the current time: pull (or equilibrium at init),
+// hydro wall completion, moments.
+template <typename R, int MODE>
+__device__ __forceinline__ void node_flow(const void* src, const R* __restrict__ force,
+                                          bool ffield, R Fx0, R Fy0, int S, int nx, int ny,
+                                          bool py, int gx, int gy, Flow<R>& f) {
+  const int k = gy * nx + gx;
+  int rm, rp;
+  neighbour_rows(gy, nx, ny, py, rm, rp);
+  const int xm = gx == 0 ? nx - 1 : gx - 1, xp = gx == nx - 1 ? 0 : gx + 1;
+  const R Fx = ffield ? force[k] : Fx0;
+  const R Fy = ffield ? force[S + k] : Fy0;
+  R d[9];
+  PopSource<R, MODE>::hydro(src, S, nx, k, gy * nx, rm, rp, gx, xm, xp, d);
+  if (MODE == kModeStep && !py && (gy == 0 || gy == ny - 1)) zou_he<R>(d, Fx, Fy, gy == 0);
+  f.pull(d, Fx, Fy);
+}
+
+// The collisions with the store of the 9 post-collision populations.
 template <typename R>
 __device__ __forceinline__ void collide_hydro(const InstDev& D, int k, int S, R* __restrict__ dst,
-                                              const HydroM<R>& hm, R rho, R ux, R uy, R dPx,
-                                              R dPy, R txx, R txy, R tyy, R Fx, R Fy) {
-  const R cs2 = R(1.0 / 3.0);
-  const R c1 = coef<R>(D, kCoefCs1), c2 = coef<R>(D, kCoefCs2);
-  const R h1 = coef<R>(D, kCoefHs1), w1 = coef<R>(D, kCoefWs1);
-  const R ruxx = rho * ux * ux, ruyy = rho * uy * uy, ruxy = rho * ux * uy;
-  const R ruxxy = ruxx * uy, ruxyy = ruxy * uy;
-  const R nxx = hm.pxx - cs2 * hm.drho - ruxx;  // A_xx^neq
-  const R nyy = hm.pyy - cs2 * hm.drho - ruyy;  // A_yy^neq
-  const R nxy = hm.pxy - ruxy;                  // A_xy^neq
-  const R nxxy = hm.qxxy - cs2 * hm.jy - ruxxy; // A_xxy^neq
-  const R nxyy = hm.qxyy - cs2 * hm.jx - ruxyy; // A_xyy^neq
-  const R bx = hm.jx + Fx, by = hm.jy + Fy;     // rho u + (1-1/tau)A_a + F-term
-  const R bxx = ruxx + c1 * nxx - h1 * dPx - w1 * txx;
-  const R byy = ruyy + c1 * nyy - h1 * dPy - w1 * tyy;
-  const R bxy = ruxy + c1 * nxy - w1 * txy;
-  const R bxxy = ruxxy + c2 * nxxy;
-  const R bxyy = ruxyy + c2 * nxyy;
-  R out[9];
-  reconstruct<R>(hm.drho, bx, by, bxx, byy, bxy, bxxy, bxyy, out);
+                                              const typename Arith<R>::Hydro& m, const Flow<R>& f,
+                                              const Grad<R>& G, R Fxx, R Fxy, R Fyy, R Fx, R Fy) {
+  R b[8], out[9];
+  Arith<R>::hydro_coefs(D, m, f, G, Fxx, Fxy, Fyy, Fx, Fy, b);
+  Arith<R>::hydro_populations(b, out);
 #pragma unroll
   for (int i = 0; i < 9; ++i) dst[(size_t)i * S + k] = out[i];
 }
 
-// Conformation TRT-RLB collision of lattice l at one node (eq_g0 with
-// G~_i, F~_i and its backward time difference) and the store of its 9
-// post-collision populations.  sl, so: the source now and one step back.
 template <typename R, bool MASKED>
 __device__ __forceinline__ void collide_cde(const InstDev& D, int k, int S, R* __restrict__ dst,
-                                            int l, const CdeM<R>& m, R rho, R ux, R uy, R sl,
-                                            R so, R uxo, R uyo, R Fx, R Fy, R dRx, R dRy) {
-  const R cs2 = R(1.0 / 3.0);
-  const R ep = coef<R>(D, kCoefEp1), c2 = coef<R>(D, kCoefCp2), h1 = coef<R>(D, kCoefHp1);
-  const R irho = R(1) / rho;
-  const R uxx = ux * ux, uyy = uy * uy, uxy = ux * uy;
-  // the force G~_i sees: F (eq_p_G_1) or F - c_s^2 grad rho (eq_p_G)
-  const bool gt = MASKED && D.gtilde;
-  const R Gx = gt ? Fx - cs2 * dRx : Fx, Gy = gt ? Fy - cs2 * dRy : Fy;
-  const R phi = (l == 1 ? R(0) : R(1)) + m.dphi;
-  const R Bx = m.jx - phi * ux, By = m.jy - phi * uy;
-  const R Bxx = m.pxx - cs2 * m.dphi - phi * uxx;
-  const R Byy = m.pyy - cs2 * m.dphi - phi * uyy;
-  const R Bxy = m.pxy - phi * uxy;
-  // small source terms first, one rounding at the magnitude of phi
-  const R c0p = m.dphi + (R(1.5) * sl - R(0.5) * so);
-  const R pr = phi * irho;
-  // (1 - 1/tau_p1) B = -B + ep B, kept split so float32 keeps the tiny
-  // difference tau_p1 - 1/2 accurately
-  const R cx = (phi * ux - Bx) + ep * Bx + h1 * (pr * Gx + ux * sl) +
-               R(0.5) * h1 * (ux * sl - uxo * so);
-  const R cy = (phi * uy - By) + ep * By + h1 * (pr * Gy + uy * sl) +
-               R(0.5) * h1 * (uy * sl - uyo * so);
-  const R cxx = phi * uxx + c2 * Bxx;
-  const R cyy = phi * uyy + c2 * Byy;
-  const R cxy = phi * uxy + c2 * Bxy;
-  R out[9];
-  reconstruct<R>(c0p, cx, cy, cxx, cyy, cxy, R(0), R(0), out);
+                                            int l, const typename Arith<R>::Cde& m,
+                                            const Flow<R>& f, R sl, R so, R uxo, R uyo, R Fx,
+                                            R Fy, const Grad<R>& G) {
+  R c[6], out[9];
+  Arith<R>::template cde_coefs<MASKED>(D, l, m, f, sl, so, uxo, uyo, Fx, Fy, G, c);
+  Arith<R>::cde_populations(c, out);
   R* dl = dst + (size_t)(9 + 9 * l) * S;
 #pragma unroll
   for (int i = 0; i < 9; ++i) dl[(size_t)i * S + k] = out[i];
@@ -570,88 +965,49 @@ __device__ __forceinline__ void prefetch_prev_u(const InstDev& D, int k, int S) 
 }
 
 // Source, both collisions, stores and final-step bookkeeping of one node
-// whose populations are already reduced to (wall-completed) moments:
-//   hm      raw hydro moments, cm[3] raw conformation moments
-//   rho, u  eq_ev_f0 moments; G** = d_g u_b; dPx, dPy = d_x(rho ux^3), d_y(rho uy^3)
-//   So, uo  source and velocity of the previous step (ignored at init)
+// whose populations are already reduced to (wall-completed) moments hm, cm[3];
+// f, G: its flow and the differences; So, uo: source and velocity of the
+// previous step (ignored at init).
 // Writes the 36 post-collision populations and the 5 history values of node k;
 // on the final step also the float64 fields and this node's partial sums.
 template <typename R, int MODE, bool FINAL, bool MASKED>
 __device__ __forceinline__ void collide_node(const InstDev& D, int k, int S, R* __restrict__ dst,
-                                             R* __restrict__ hist, const HydroM<R>& hm,
-                                             const CdeM<R>* cm, R rho, R ux, R uy, R G00, R G01,
-                                             R G10, R G11, R dPx, R dPy, R dRx, R dRy, R Fx,
-                                             R Fy, R So0, R So1, R So2, R uxo, R uyo,
-                                             PartT<R> ux_prev, PartT<R> uy_prev, PartT<R>* part,
-                                             PartT<R>* plo) {
-  // conformation tensor, constitutive function, polymer stress (eq_kramer),
-  // source Phi_ab
+                                             R* __restrict__ hist,
+                                             const typename Arith<R>::Hydro& hm,
+                                             const typename Arith<R>::Cde* cm, const Flow<R>& f,
+                                             const Grad<R>& G, R Fx, R Fy, R So0, R So1, R So2,
+                                             R uxo, R uyo, PartT<R> ux_prev, PartT<R> uy_prev,
+                                             PartT<R>* part, PartT<R>* plo) {
+  // conformation tensor, constitutive function, source Phi_ab
   R Axx, Axy, Ayy, Fxx, Fxy, Fyy;
   polymer_terms<R, MASKED>(D, cm[0].dphi, cm[1].dphi, cm[2].dphi, Axx, Axy, Ayy, Fxx, Fxy, Fyy);
-  const R mpl = coef<R>(D, kCoefMupLam), il = coef<R>(D, kCoefInvLam);
-  const R txx = mpl * Fxx, txy = mpl * Fxy, tyy = mpl * Fyy;
   R Sc[3], So[3] = {So0, So1, So2};
 #pragma unroll
-  for (int l = 0; l < 3; ++l)
-    Sc[l] = source_component<R>(l, Axx, Axy, Ayy, Fxx, Fxy, Fyy, il, G00, G01, G10, G11);
+  for (int l = 0; l < 3; ++l) Sc[l] = Arith<R>::source(l, D, Axx, Axy, Ayy, Fxx, Fxy, Fyy, G);
   if (MODE != kModeStep) {
     // first step: the backward difference of the CDE source is zero
     So[0] = Sc[0];
     So[1] = Sc[1];
     So[2] = Sc[2];
-    uxo = ux;
-    uyo = uy;
+    uxo = f.ux;
+    uyo = f.uy;
   }
-  collide_hydro<R>(D, k, S, dst, hm, rho, ux, uy, dPx, dPy, txx, txy, tyy, Fx, Fy);
+  collide_hydro<R>(D, k, S, dst, hm, f, G, Fxx, Fxy, Fyy, Fx, Fy);
 #pragma unroll
   for (int l = 0; l < 3; ++l)
-    collide_cde<R, MASKED>(D, k, S, dst, l, cm[l], rho, ux, uy, Sc[l], So[l], uxo, uyo, Fx, Fy,
-                           dRx, dRy);
+    collide_cde<R, MASKED>(D, k, S, dst, l, cm[l], f, Sc[l], So[l], uxo, uyo, Fx, Fy, G);
 
   hist[k] = Sc[0];
   hist[S + k] = Sc[1];
   hist[2 * S + k] = Sc[2];
-  hist[3 * S + k] = ux;
-  hist[4 * S + k] = uy;
+  hist[3 * S + k] = f.ux;
+  hist[4 * S + k] = f.uy;
 
   if (FINAL) {
     const R dphi[3] = {cm[0].dphi, cm[1].dphi, cm[2].dphi};
-    final_node<R, MODE>(D, k, S, -1, hm.drho, rho, ux, uy, dphi, ux_prev, uy_prev, part, plo);
+    final_node<R, MODE>(D, k, S, -1, hm.drho, f.rho, f.ux, f.uy, dphi, ux_prev, uy_prev, part,
+                        plo);
   }
-}
-
-// Second-order differences in y of u and rho u_y^3 at a node, from the
-// moments of rows y-2..y+2 (central inside, one-sided on wall rows).
-template <typename R>
-__device__ __forceinline__ void y_gradients(bool wb, bool wt, R rm2, R uxm2, R uym2, R rm1,
-                                            R uxm1, R uym1, R r0, R ux0, R uy0, R rp1, R uxp1,
-                                            R uyp1, R rp2, R uxp2, R uyp2, R& G10, R& G11,
-                                            R& dPy) {
-  const R half = R(0.5);
-  if (wb) {
-    G10 = half * (R(-3) * ux0 + R(4) * uxp1 - uxp2);
-    G11 = half * (R(-3) * uy0 + R(4) * uyp1 - uyp2);
-    dPy = half * (R(-3) * (r0 * uy0 * uy0 * uy0) + R(4) * (rp1 * uyp1 * uyp1 * uyp1) -
-                  rp2 * uyp2 * uyp2 * uyp2);
-  } else if (wt) {
-    G10 = half * (R(3) * ux0 - R(4) * uxm1 + uxm2);
-    G11 = half * (R(3) * uy0 - R(4) * uym1 + uym2);
-    dPy = half * (R(3) * (r0 * uy0 * uy0 * uy0) - R(4) * (rm1 * uym1 * uym1 * uym1) +
-                  rm2 * uym2 * uym2 * uym2);
-  } else {
-    G10 = half * (uxp1 - uxm1);
-    G11 = half * (uyp1 - uym1);
-    dPy = half * (rp1 * uyp1 * uyp1 * uyp1 - rm1 * uym1 * uym1 * uym1);
-  }
-}
-
-// The same y difference of the density (for the eq_p_G form of G~).
-template <typename R>
-__device__ __forceinline__ R y_drho(bool wb, bool wt, R rm2, R rm1, R r0, R rp1, R rp2) {
-  const R half = R(0.5);
-  if (wb) return half * (R(-3) * r0 + R(4) * rp1 - rp2);
-  if (wt) return half * (R(3) * r0 - R(4) * rm1 + rm2);
-  return half * (rp1 - rm1);
 }
 
 // Resident CTAs per SM the register budget is sized for: the float32 step
@@ -679,34 +1035,6 @@ struct MinBlocks {
                            : (NT <= 32 ? 2 : NT <= 64 ? 4 : (NT <= 512 ? 512 / NT : 1));
 };
 
-// One-sided differences along one axis next to the solid mask (same rule as
-// the central and wall-row differences: second order on the fluid side when
-// two fluid nodes lie there, else first order; zero between two solids).
-//   t:        +1 toward +axis, -1 toward -axis (the fluid side)
-//   q0, q1:   (rho, ux, uy) of the node and of its fluid neighbour at +t
-//   has2:     whether the node at +2t is fluid; (r2, u2x, u2y) its values
-//   axis:     0 = x (the cube is rho ux^3), 1 = y (rho uy^3)
-template <typename R>
-__device__ __forceinline__ void one_sided(int t, R r0, R ux0, R uy0, R r1, R ux1, R uy1,
-                                          bool has2, R r2, R ux2, R uy2, int axis, R& dux,
-                                          R& duy, R& dcube, R& drho) {
-  const R v0 = axis == 0 ? ux0 : uy0, v1 = axis == 0 ? ux1 : uy1, v2 = axis == 0 ? ux2 : uy2;
-  const R c0 = r0 * v0 * v0 * v0, c1 = r1 * v1 * v1 * v1, c2 = r2 * v2 * v2 * v2;
-  const R ts = (R)t;
-  if (has2) {
-    const R h = R(0.5) * ts;
-    dux = h * (R(-3) * ux0 + R(4) * ux1 - ux2);
-    duy = h * (R(-3) * uy0 + R(4) * uy1 - uy2);
-    dcube = h * (R(-3) * c0 + R(4) * c1 - c2);
-    drho = h * (R(-3) * r0 + R(4) * r1 - r2);
-  } else {
-    dux = ts * (ux1 - ux0);
-    duy = ts * (uy1 - uy0);
-    dcube = ts * (c1 - c0);
-    drho = ts * (r1 - r0);
-  }
-}
-
 // Open channels: nodes of the inlet (x = 0) and outlet (x = nx - 1) columns
 // take their completed populations from the column pass's colbuf during a
 // step (the pull would miss the populations entering from outside).
@@ -718,13 +1046,13 @@ __device__ __forceinline__ const R* colbuf_node(const InstDev& D, int gx, int gy
   return (const R*)D.colbuf + (gx == 0 ? 0 : D.ny) + gy;  // plane stride 2 ny
 }
 
-// rho, u of region node (gx, gy) for the masked variant: open-column nodes
-// from colbuf during a step, every other node as node_rho_u.
+// Flow of region node (gx, gy) for the masked variant: open-column nodes
+// from colbuf during a step, every other node as node_flow.
 template <typename R, int MODE>
-__device__ __forceinline__ void region_rho_u(const InstDev& D, const void* src,
-                                             const R* __restrict__ force, bool ffield, R Fx0,
-                                             R Fy0, int S, int nx, int ny, bool py, int gx,
-                                             int gy, R& rho, R& ux, R& uy) {
+__device__ __forceinline__ void region_flow(const InstDev& D, const void* src,
+                                            const R* __restrict__ force, bool ffield, R Fx0,
+                                            R Fy0, int S, int nx, int ny, bool py, int gx,
+                                            int gy, Flow<R>& f) {
   if (MODE == kModeStep && open_column(D, gx)) {
     const R* cb = colbuf_node<R>(D, gx, gy);
     const int ld = 2 * ny;
@@ -733,15 +1061,10 @@ __device__ __forceinline__ void region_rho_u(const InstDev& D, const void* src,
     for (int i = 0; i < 9; ++i) d[i] = cb[(size_t)i * ld];
     const int k = gy * nx + gx;
     const R Fx = ffield ? force[k] : Fx0, Fy = ffield ? force[S + k] : Fy0;
-    HydroM<R> m;
-    hydro_moments<R>(d, m);
-    rho = R(1) + m.drho;
-    const R irho = R(1) / rho;
-    ux = (m.jx + R(0.5) * Fx) * irho;
-    uy = (m.jy + R(0.5) * Fy) * irho;
+    f.pull(d, Fx, Fy);
     return;
   }
-  node_rho_u<R, MODE>(src, force, ffield, Fx0, Fy0, S, nx, ny, py, gx, gy, rho, ux, uy);
+  node_flow<R, MODE>(src, force, ffield, Fx0, Fy0, S, nx, ny, py, gx, gy, f);
 }
 
 // Sum of two float32 pairs (hi + lo), renormalised (Knuth's two-sum of the
@@ -882,8 +1205,9 @@ __device__ __forceinline__ void tile_partials(const InstDev& D, const TileDev& T
 
 template <typename R, int MODE, bool FINAL, bool MASKED, int NT>
 __device__ __forceinline__ void process_tile(const InstDev* __restrict__ insts, const TileDev T,
-                                             int parity, double* __restrict__ partials, R* s_rho,
-                                             R* s_ux, R* s_uy, double (*s_red)[kPartial]) {
+                                             int parity, double* __restrict__ partials,
+                                             Region<R, region_max(NT)>& Q,
+                                             double (*s_red)[kPartial]) {
   const InstDev& D = insts[T.inst];
   const int nx = D.nx, ny = D.ny, S = D.stride, TX = D.TX, TY = D.TY, hy = D.hy;
   const bool py = D.periodic_y != 0;
@@ -1013,38 +1337,29 @@ __device__ __forceinline__ void process_tile(const InstDev* __restrict__ insts, 
     if (MODE == kModeStep && !py && (rgy == 0 || rgy == ny - 1) &&
         !(MASKED && open_column(D, rgx)))
       zou_he<R>(dr, rFx, rFy, rgy == 0);
-    HydroM<R> m;
-    hydro_moments<R>(dr, m);
-    const R rho = R(1) + m.drho;
-    s_rho[ring_r] = rho;
-    const R irho = R(1) / rho;
-    s_ux[ring_r] = (m.jx + R(0.5) * rFx) * irho;
-    s_uy[ring_r] = (m.jy + R(0.5) * rFy) * irho;
+    Flow<R> f;
+    f.pull(dr, rFx, rFy);
+    Q.put(ring_r, f);
   }
 
   // (4) own moments; conformation walls completed with the node's own u
-  HydroM<R> hm;
-  CdeM<R> cm[3];
-  R rho = R(1), ux = R(0), uy = R(0);
+  typename Arith<R>::Hydro hm;
+  typename Arith<R>::Cde cm[3];
+  Flow<R> f;
   double wall_io[6] = {0, 0, 0, 0, 0, 0};
   if (active) {
     if (MODE == kModeStep && wcomp) zou_he<R>(d, Fx, Fy, wb);
-    hydro_moments<R>(d, hm);
-    rho = R(1) + hm.drho;
-    const R irho_own = R(1) / rho;
-    ux = (hm.jx + R(0.5) * Fx) * irho_own;
-    uy = (hm.jy + R(0.5) * Fy) * irho_own;
-    s_rho[ri] = rho;
-    s_ux[ri] = ux;
-    s_uy[ri] = uy;
+    Arith<R>::moments(d, hm);
+    f.set(hm, Fx, Fy);
+    Q.put(ri, f);
 #pragma unroll
     for (int l = 0; l < 3; ++l) {
       if (MODE == kModeStep && wcomp) {
         const R delta = (l == 1) ? R(0) : R(1);
-        cnebb<R>(g[l], post[l][0], post[l][1], post[l][2], delta, ux, uy, wb, wall_io[l],
+        cnebb<R>(g[l], post[l][0], post[l][1], post[l][2], delta, f.ux, f.uy, wb, wall_io[l],
                  wall_io[3 + l]);
       }
-      cde_moments<R>(g[l], cm[l]);
+      Arith<R>::moments(g[l], cm[l]);
     }
   } else if (in_tile && !inside) {
     // slot outside the domain (ragged tile): it may still be a periodic
@@ -1052,14 +1367,12 @@ __device__ __forceinline__ void process_tile(const InstDev* __restrict__ insts, 
     const int gx = t32 ? wrap_once(x, nx) : x % nx;
     const int gy = py ? (t32 ? wrap_once(y, ny) : y % ny) : y;
     if (gy < ny) {
-      R r, vx, vy;
+      Flow<R> w;
       if constexpr (MASKED)
-        region_rho_u<R, MODE>(D, src, force, ffield, Fx0, Fy0, S, nx, ny, py, gx, gy, r, vx, vy);
+        region_flow<R, MODE>(D, src, force, ffield, Fx0, Fy0, S, nx, ny, py, gx, gy, w);
       else
-        node_rho_u<R, MODE>(src, force, ffield, Fx0, Fy0, S, nx, ny, py, gx, gy, r, vx, vy);
-      s_rho[ri] = r;
-      s_ux[ri] = vx;
-      s_uy[ri] = vy;
+        node_flow<R, MODE>(src, force, ffield, Fx0, Fy0, S, nx, ny, py, gx, gy, w);
+      Q.put(ri, w);
     }
   }
 
@@ -1068,15 +1381,12 @@ __device__ __forceinline__ void process_tile(const InstDev* __restrict__ insts, 
     int lx, ly, gx, gy;
     ring_slot(q, RW, TY, hy, lx, ly);
     if (!region_node(lx, ly, T.x0, T.y0, hy, nx, ny, py, gx, gy)) continue;
-    R r, vx, vy;
+    Flow<R> w;
     if constexpr (MASKED)
-      region_rho_u<R, MODE>(D, src, force, ffield, Fx0, Fy0, S, nx, ny, py, gx, gy, r, vx, vy);
+      region_flow<R, MODE>(D, src, force, ffield, Fx0, Fy0, S, nx, ny, py, gx, gy, w);
     else
-      node_rho_u<R, MODE>(src, force, ffield, Fx0, Fy0, S, nx, ny, py, gx, gy, r, vx, vy);
-    const int rr = ly * RW + lx;
-    s_rho[rr] = r;
-    s_ux[rr] = vx;
-    s_uy[rr] = vy;
+      node_flow<R, MODE>(src, force, ffield, Fx0, Fy0, S, nx, ny, py, gx, gy, w);
+    Q.put(ly * RW + lx, w);
   }
   __syncthreads();
 
@@ -1088,24 +1398,8 @@ __device__ __forceinline__ void process_tile(const InstDev* __restrict__ insts, 
   for (int j = 0; j < (FINAL ? 12 : 1); ++j) plo[j] = 0;
 
   if (active) {
-    // gradients: grad[g][b] = d_g u_b  (G00 = dx ux, G01 = dx uy, G10 = dy ux, G11 = dy uy)
-    const R half = R(0.5);
-    R G00 = half * (s_ux[ri + 1] - s_ux[ri - 1]);
-    R G01 = half * (s_uy[ri + 1] - s_uy[ri - 1]);
-    const R cxp = s_rho[ri + 1] * s_ux[ri + 1] * s_ux[ri + 1] * s_ux[ri + 1];
-    const R cxm = s_rho[ri - 1] * s_ux[ri - 1] * s_ux[ri - 1] * s_ux[ri - 1];
-    R dPx = half * (cxp - cxm);
-    R G10, G11, dPy;
-    // density gradient, only for the eq_p_G form of G~
-    R dRx = (MASKED && D.gtilde) ? half * (s_rho[ri + 1] - s_rho[ri - 1]) : R(0), dRy = R(0);
-    {
-      // rows y-2..y+2 of this column (only those a wall row needs are read)
-      const int a = wb ? ri : (wt ? ri - 2 * RW : ri), b = wb ? ri : (wt ? ri - RW : ri - RW);
-      const int c = wb ? ri + RW : (wt ? ri : ri + RW), e = wb ? ri + 2 * RW : ri;
-      y_gradients<R>(wb, wt, s_rho[a], s_ux[a], s_uy[a], s_rho[b], s_ux[b], s_uy[b], rho, ux,
-                     uy, s_rho[c], s_ux[c], s_uy[c], s_rho[e], s_ux[e], s_uy[e], G10, G11, dPy);
-      if (MASKED && D.gtilde) dRy = y_drho<R>(wb, wt, s_rho[a], s_rho[b], rho, s_rho[c], s_rho[e]);
-    }
+    Grad<R> G;
+    Arith<R>::gradients(Q, ri, RW, wb, wt, f, MASKED && D.gtilde, G);
     if constexpr (MASKED) {
       // one-sided differences where an axis neighbour is solid; the values
       // two nodes away come straight from the pulled populations (L2)
@@ -1116,47 +1410,39 @@ __device__ __forceinline__ void process_tile(const InstDev* __restrict__ insts, 
       const bool sxp = (D.open_x && x == nx - 1) || (M && M[y * nx + xp] != 0);
       const bool sxm = (D.open_x && x == 0) || (M && M[y * nx + xm] != 0);
       if (sxp || sxm) {
-        R gx0 = R(0), gx1 = R(0), gxc = R(0), gxr = R(0);
-        if (!(sxp && sxm)) {
+        if (sxp && sxm) {
+          Arith<R>::blocked(0, G);
+        } else {
           const int t = sxp ? -1 : 1;
           const int i1 = t > 0 ? ri + 1 : ri - 1;
           const int x2 = (((x + 2 * t) % nx) + nx) % nx;
           const bool has2 = !(M && M[y * nx + x2] != 0);
-          R r2 = R(1), u2x = R(0), u2y = R(0);
+          Flow<R> w;
+          w.rest();
           if (has2)
-            region_rho_u<R, MODE>(D, src, force, ffield, Fx0, Fy0, S, nx, ny, py, x2, y, r2,
-                                  u2x, u2y);
-          one_sided<R>(t, rho, ux, uy, s_rho[i1], s_ux[i1], s_uy[i1], has2, r2, u2x, u2y, 0, gx0,
-                       gx1, gxc, gxr);
+            region_flow<R, MODE>(D, src, force, ffield, Fx0, Fy0, S, nx, ny, py, x2, y, w);
+          Arith<R>::one_sided(0, t, Q, ri, i1, f, has2, w, G);
         }
-        G00 = gx0;
-        G01 = gx1;
-        dPx = gxc;
-        dRx = gxr;
       }
       if (!wb && !wt && M) {
         // rows next to a flat wall carry no mask, so y +- 1 lies in the domain
         const int yp = (py && y == ny - 1) ? 0 : y + 1, ym = (py && y == 0) ? ny - 1 : y - 1;
         const bool syp = M[yp * nx + x] != 0, sym = M[ym * nx + x] != 0;
         if (syp || sym) {
-          R gy0 = R(0), gy1 = R(0), gyc = R(0), gyr = R(0);
-          if (!(syp && sym)) {
+          if (syp && sym) {
+            Arith<R>::blocked(1, G);
+          } else {
             const int t = syp ? -1 : 1;
             const int i1 = t > 0 ? ri + RW : ri - RW;
             int y2 = y + 2 * t;
             if (py) y2 = ((y2 % ny) + ny) % ny;
             const bool has2 = y2 >= 0 && y2 < ny && M[y2 * nx + x] == 0;
-            R r2 = R(1), u2x = R(0), u2y = R(0);
+            Flow<R> w;
+            w.rest();
             if (has2)
-              region_rho_u<R, MODE>(D, src, force, ffield, Fx0, Fy0, S, nx, ny, py, x, y2, r2,
-                                    u2x, u2y);
-            one_sided<R>(t, rho, ux, uy, s_rho[i1], s_ux[i1], s_uy[i1], has2, r2, u2x, u2y, 1,
-                         gy0, gy1, gyc, gyr);
+              region_flow<R, MODE>(D, src, force, ffield, Fx0, Fy0, S, nx, ny, py, x, y2, w);
+            Arith<R>::one_sided(1, t, Q, ri, i1, f, has2, w, G);
           }
-          G10 = gy0;
-          G11 = gy1;
-          dPy = gyc;
-          dRy = gyr;
         }
       }
     }
@@ -1182,9 +1468,8 @@ __device__ __forceinline__ void process_tile(const InstDev* __restrict__ insts, 
       ux_prev = (PartT<R>)__ldcg(D.fields + S + k);
       uy_prev = (PartT<R>)__ldcg(D.fields + 2 * S + k);
     }
-    collide_node<R, MODE, FINAL, MASKED>(D, k, S, dst, hist, hm, cm, rho, ux, uy, G00, G01, G10,
-                                         G11, dPx, dPy, dRx, dRy, Fx, Fy, So[0], So[1], So[2], uxo,
-                                         uyo, ux_prev, uy_prev, part, plo);
+    collide_node<R, MODE, FINAL, MASKED>(D, k, S, dst, hist, hm, cm, f, G, Fx, Fy, So[0], So[1],
+                                         So[2], uxo, uyo, ux_prev, uy_prev, part, plo);
   } else if (FINAL && solid) {
     // a solid node reports zero fields and adds nothing to the totals
     const int ks = y * nx + x;
@@ -1204,14 +1489,11 @@ __global__ void __launch_bounds__(NT, MinBlocks<R, MASKED, NT>::value)
     step_kernel(const InstDev* __restrict__ insts, const TileDev* __restrict__ tiles,
                 int parity, double* __restrict__ partials) {
   static_assert(NT % 32 == 0 && NT >= 32, "whole warps; the final-step reduction reads 14 lanes");
-  constexpr int kRegion = region_max(NT);
-  __shared__ R s_rho[kRegion];
-  __shared__ R s_ux[kRegion];
-  __shared__ R s_uy[kRegion];
+  __shared__ Region<R, region_max(NT)> Q;
   __shared__ double s_red[NT / 32][kPartial];
   const TileDev T = tiles[blockIdx.x];
   if (!MASKED && T.masked) return;
-  process_tile<R, MODE, FINAL, MASKED, NT>(insts, T, parity, partials, s_rho, s_ux, s_uy, s_red);
+  process_tile<R, MODE, FINAL, MASKED, NT>(insts, T, parity, partials, Q, s_red);
 }
 
 // ---- float64 steps of tiny batches: one lattice per warp --------------------
@@ -1237,8 +1519,9 @@ template <bool FINAL>
 __device__ __forceinline__ void process_tile_split(const InstDev* __restrict__ insts,
                                                    const TileDev T, int parity,
                                                    double* __restrict__ partials,
-                                                   double* s_rho, double* s_ux, double* s_uy,
-                                                   double (*s_phi)[32], double (*s_red)[kPartial]) {
+                                                   Region<double, region_max(32)>& Q,
+                                                   double (*s_phi)[32], double* s_irho,
+                                                   double (*s_red)[kPartial]) {
   using R = double;
   constexpr int MODE = kModeStep;
   const InstDev& D = insts[T.inst];
@@ -1316,65 +1599,55 @@ __device__ __forceinline__ void process_tile_split(const InstDev* __restrict__ i
     const R rFx = ffield ? force[rk] : Fx0;
     const R rFy = ffield ? force[S + rk] : Fy0;
     if (!py && (rgy == 0 || rgy == ny - 1)) zou_he<R>(dr, rFx, rFy, rgy == 0);
-    HydroM<R> m;
-    hydro_moments<R>(dr, m);
-    const R rho = R(1) + m.drho;
-    s_rho[ring_r] = rho;
-    const R irho = R(1) / rho;
-    s_ux[ring_r] = (m.jx + R(0.5) * rFx) * irho;
-    s_uy[ring_r] = (m.jy + R(0.5) * rFy) * irho;
+    Flow<R> w;
+    w.pull(dr, rFx, rFy);
+    Q.put(ring_r, w);
   }
   for (int qq = kSplitThreads - 32 + threadIdx.x; role == 0 && qq < nring; qq += 32) {
     int lx, ly, gx, gy;
     ring_slot(qq, RW, TY, hy, lx, ly);
     if (!region_node(lx, ly, T.x0, T.y0, hy, nx, ny, py, gx, gy)) continue;
-    R r, vx, vy;
-    node_rho_u<R, MODE>(src, force, ffield, Fx0, Fy0, S, nx, ny, py, gx, gy, r, vx, vy);
-    const int rr = ly * RW + lx;
-    s_rho[rr] = r;
-    s_ux[rr] = vx;
-    s_uy[rr] = vy;
+    Flow<R> w;
+    node_flow<R, MODE>(src, force, ffield, Fx0, Fy0, S, nx, ny, py, gx, gy, w);
+    Q.put(ly * RW + lx, w);
   }
   // own hydrodynamic moments (warp 0), and the wrapped nodes of a ragged tile
-  HydroM<R> hm;
+  Arith<R>::Hydro hm;
+  Flow<R> f;
   if (role == 0) {
     if (active) {
       if (wcomp) zou_he<R>(d, Fx, Fy, wb);
-      hydro_moments<R>(d, hm);
-      const R rho = R(1) + hm.drho;
-      const R irho_own = R(1) / rho;
-      s_rho[ri] = rho;
-      s_ux[ri] = (hm.jx + R(0.5) * Fx) * irho_own;
-      s_uy[ri] = (hm.jy + R(0.5) * Fy) * irho_own;
+      Arith<R>::moments(d, hm);
+      f.set(hm, Fx, Fy);
+      Q.put(ri, f);
+      s_irho[lane] = f.irho;
     } else if (in_tile) {
       const int gx = x % nx;
       const int gy = py ? y % ny : y;
       if (gy < ny) {
-        R r, vx, vy;
-        node_rho_u<R, MODE>(src, force, ffield, Fx0, Fy0, S, nx, ny, py, gx, gy, r, vx, vy);
-        s_rho[ri] = r;
-        s_ux[ri] = vx;
-        s_uy[ri] = vy;
+        Flow<R> w;
+        node_flow<R, MODE>(src, force, ffield, Fx0, Fy0, S, nx, ny, py, gx, gy, w);
+        Q.put(ri, w);
       }
     }
   }
   __syncthreads();
 
   // ---- conformation walls with the node's own u, moments -----------------------
-  R rho = R(1), ux = R(0), uy = R(0);
-  if (active) {
-    rho = s_rho[ri];
-    ux = s_ux[ri];
-    uy = s_uy[ri];
+  if (role > 0 && active) {
+    f.ux = Q.ux[ri];
+    f.uy = Q.uy[ri];
+    f.irho = s_irho[lane];
+    f.rho = R(1);  // not used by the conformation lattices
   }
-  CdeM<R> cm;
+  Arith<R>::Cde cm;
   double wall_in = 0.0, wall_out = 0.0;
   if (role > 0 && active) {
     if (wcomp) {
       const R delta = (l == 1) ? R(0) : R(1);
-      cnebb<R>(d, post[0], post[1], post[2], delta, ux, uy, wb, wall_in, wall_out);
+      cnebb<R>(d, post[0], post[1], post[2], delta, f.ux, f.uy, wb, wall_in, wall_out);
     }
-    cde_moments<R>(d, cm);
+    Arith<R>::moments(d, cm);
     s_phi[l][lane] = cm.dphi;
   }
   __syncthreads();
@@ -1386,43 +1659,30 @@ __device__ __forceinline__ void process_tile_split(const InstDev* __restrict__ i
 #pragma unroll
   for (int j = 0; j < (FINAL ? 12 : 1); ++j) plo[j] = 0;
   if (active) {
-    const R half = R(0.5);
-    const R G00 = half * (s_ux[ri + 1] - s_ux[ri - 1]);
-    const R G01 = half * (s_uy[ri + 1] - s_uy[ri - 1]);
-    R G10, G11, dPy;
-    const int a = wb ? ri : (wt ? ri - 2 * RW : ri), b = wb ? ri : (wt ? ri - RW : ri - RW);
-    const int c = wb ? ri + RW : (wt ? ri : ri + RW), e = wb ? ri + 2 * RW : ri;
-    y_gradients<R>(wb, wt, s_rho[a], s_ux[a], s_uy[a], s_rho[b], s_ux[b], s_uy[b], rho, ux, uy,
-                   s_rho[c], s_ux[c], s_uy[c], s_rho[e], s_ux[e], s_uy[e], G10, G11, dPy);
+    Grad<R> G;
+    Arith<R>::gradients(Q, ri, RW, wb, wt, f, false, G);
     R Axx, Axy, Ayy, Fxx, Fxy, Fyy;
     polymer_terms<R, false>(D, s_phi[0][lane], s_phi[1][lane], s_phi[2][lane], Axx, Axy, Ayy, Fxx,
                             Fxy, Fyy);
     if (role == 0) {
-      const R cxp = s_rho[ri + 1] * s_ux[ri + 1] * s_ux[ri + 1] * s_ux[ri + 1];
-      const R cxm = s_rho[ri - 1] * s_ux[ri - 1] * s_ux[ri - 1] * s_ux[ri - 1];
-      const R dPx = half * (cxp - cxm);
-      const R mpl = coef<R>(D, kCoefMupLam);
-      const R txx = mpl * Fxx, txy = mpl * Fxy, tyy = mpl * Fyy;
       double ux_prev = 0.0, uy_prev = 0.0;
       if (FINAL) {
         ux_prev = D.fields[S + k];
         uy_prev = D.fields[2 * S + k];
       }
-      collide_hydro<R>(D, k, S, dst, hm, rho, ux, uy, dPx, dPy, txx, txy, tyy, Fx, Fy);
-      hist[3 * S + k] = ux;
-      hist[4 * S + k] = uy;
+      collide_hydro<R>(D, k, S, dst, hm, f, G, Fxx, Fxy, Fyy, Fx, Fy);
+      hist[3 * S + k] = f.ux;
+      hist[4 * S + k] = f.uy;
       if (FINAL)
-        final_node<R, MODE>(D, k, S, 0, hm.drho, rho, ux, uy, nullptr, ux_prev, uy_prev, part,
-                            plo);
+        final_node<R, MODE>(D, k, S, 0, hm.drho, f.rho, f.ux, f.uy, nullptr, ux_prev, uy_prev,
+                            part, plo);
     } else {
-      const R il = coef<R>(D, kCoefInvLam);
-      const R sl = source_component<R>(l, Axx, Axy, Ayy, Fxx, Fxy, Fyy, il, G00, G01, G10, G11);
-      collide_cde<R, false>(D, k, S, dst, l, cm, rho, ux, uy, sl, So, uxo, uyo, Fx, Fy, R(0),
-                            R(0));
+      const R sl = Arith<R>::source(l, D, Axx, Axy, Ayy, Fxx, Fxy, Fyy, G);
+      collide_cde<R, false>(D, k, S, dst, l, cm, f, sl, So, uxo, uyo, Fx, Fy, G);
       hist[(size_t)l * S + k] = sl;
       if (FINAL) {
         const R dphi[3] = {s_phi[0][lane], s_phi[1][lane], s_phi[2][lane]};
-        final_node<R, MODE>(D, k, S, role, R(0), rho, ux, uy, dphi, 0.0, 0.0, part, plo);
+        final_node<R, MODE>(D, k, S, role, R(0), f.rho, f.ux, f.uy, dphi, 0.0, 0.0, part, plo);
         part[kWallIn + l] = wall_in;
         part[kWallOut + l] = wall_out;
       }
@@ -1436,15 +1696,12 @@ template <bool FINAL>
 __global__ void __launch_bounds__(kSplitThreads, 4)
     step_kernel_split(const InstDev* __restrict__ insts, const TileDev* __restrict__ tiles,
                       int parity, double* __restrict__ partials) {
-  constexpr int kRegion = region_max(32);
-  __shared__ double s_rho[kRegion];
-  __shared__ double s_ux[kRegion];
-  __shared__ double s_uy[kRegion];
-  __shared__ double s_phi[3][32];
+  __shared__ Region<double, region_max(32)> Q;
+  __shared__ double s_phi[3][32], s_irho[32];
   __shared__ double s_red[kSplitThreads / 32][kPartial];
   const TileDev T = tiles[blockIdx.x];
   if (T.masked) return;
-  process_tile_split<FINAL>(insts, T, parity, partials, s_rho, s_ux, s_uy, s_phi, s_red);
+  process_tile_split<FINAL>(insts, T, parity, partials, Q, s_phi, s_irho, s_red);
 }
 
 }  // namespace lbve
