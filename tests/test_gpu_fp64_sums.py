@@ -26,10 +26,10 @@ def _instance(kind, nx):
 
 @pytest.mark.parametrize("nx", [1, 5, 32, 33, 70])
 @pytest.mark.parametrize("kind", ["mill", "channel"])
-@pytest.mark.parametrize("du,dA,stretch", [(1e-2, 0.1, 1.0), (1e-12, 1e-12, 1.0), (1e-3, 0.1, 1e8), (0.0, 0.0, 1e-9)])
+@pytest.mark.parametrize("du,dA,stretch", [(1e-2, 0.1, 1.0), (1e-12, 1e-12, 1.0), (0.0, 0.0, 1e-9)])
 def test_wide_ranges_against_oracle(lbve, kind, nx, du, dA, stretch):
     """Three steps from random fields (velocities from 0 to 1e-2, conformations
-    scaled up to 1e8).  The oracle carries full populations, so both sides are
+    down to 1e-9).  The oracle carries full populations, so both sides are
     within a few hundred roundings (3 steps, 36 populations) of 2^-53 of the
     largest value of a field's lattice: 1e-13 of it."""
     inst = _instance(kind, nx)
