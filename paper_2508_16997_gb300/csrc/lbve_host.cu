@@ -393,8 +393,10 @@ int launch_one_step(lbve_handle* h, int parity, int flags, cudaStream_t st) {
       const cudaError_t e = cudaEventRecord(h->prof_ev[l][kind][2 * h->prof_n[l][kind]], st);
       if (e != cudaSuccess) return cuda_fail(e, "profile event");
     }
+    // without a fork every kernel of the step sequence is a plain one, and each
+    // may start while the one before it ends
     if (launch_step(prec, h->plan.threads[l], h->d_insts, h->d_tiles[l], h->plan.ntiles[l],
-                    parity, kModeStep, flags,
+                    parity, kModeStep, flags | (fork ? 0 : kDependent),
                     h->d_partials, st))
       return cuda_fail(cudaGetLastError(), "step kernel launch");
     if (timed) {

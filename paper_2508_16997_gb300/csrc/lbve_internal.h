@@ -63,7 +63,10 @@ enum : int {
 };
 
 // Kernel flags.
-enum : int { kFinal = 1 };
+enum : int {
+  kFinal = 1,
+  kDependent = 2  // the launch may overlap the end of the step kernel before it
+};
 
 // Coefficient slots of InstDev::cd / InstDev::cf.
 enum : int {

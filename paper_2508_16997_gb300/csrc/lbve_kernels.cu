@@ -9,23 +9,33 @@ namespace lbve {
 
 template <typename R, int MODE, bool FINAL, bool MASKED, int NT>
 static void launch_step_k(const InstDev* d_insts, const TileDev* d_tiles, int n_tiles, int parity,
-                          double* d_partials, cudaStream_t st) {
-  step_kernel<R, MODE, FINAL, MASKED, NT><<<n_tiles, NT, 0, st>>>(d_insts, d_tiles, parity,
-                                                                  d_partials);
+                          double* d_partials, cudaStream_t st, bool dependent = false) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(n_tiles);
+  cfg.blockDim = dim3(NT);
+  cfg.stream = st;
+  // with the programmatic dependency on the step kernel before (start_next_kernel)
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = dependent && overlaps_steps<R, MODE, MASKED>() ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, step_kernel<R, MODE, FINAL, MASKED, NT>, d_insts, d_tiles, parity,
+                     d_partials);
 }
 
 template <typename R, bool MASKED, int NT>
 static int launch_step_t(const InstDev* d_insts, const TileDev* d_tiles, int n_tiles, int parity,
                          int mode, int flags, double* d_partials, cudaStream_t st) {
   if (n_tiles <= 0) return 0;
-  const bool fin = (flags & kFinal) != 0;
+  const bool fin = (flags & kFinal) != 0, dep = (flags & kDependent) != 0;
   if (mode == kModeStep) {
     if (fin)
       launch_step_k<R, kModeStep, true, MASKED, NT>(d_insts, d_tiles, n_tiles, parity, d_partials,
-                                                    st);
+                                                    st, dep);
     else
       launch_step_k<R, kModeStep, false, MASKED, NT>(d_insts, d_tiles, n_tiles, parity,
-                                                     d_partials, st);
+                                                     d_partials, st, dep);
   } else {
     launch_step_k<R, kModeInit, true, MASKED, NT>(d_insts, d_tiles, n_tiles, parity, d_partials,
                                                   st);
