@@ -145,10 +145,13 @@ struct Plan {
   int ncols[kLists];      // open-column tasks per list
 };
 
-// Default tile width: 32 (one warp along x), or 8 for the one-warp float64
-// CTAs, whose 8 x 4 tiles have a third of the halo ring of 32 x 1 tiles.
+// Default tile width: 32 (one warp along x), or 8 for the one- and two-warp
+// float64 CTAs: 8 x 4 tiles have a third of the halo ring of 32 x 1 tiles, and
+// the ring of an 8 x 8 tile (32 nodes, 48 at walls) is one round of its 64
+// threads where that of a 32 x 2 tile (68, 132) takes two or three (128^2 mill
+// 15.3 -> 13.3 us per step, 192^2 21.2 -> 19.3).
 int default_tile_tx(const lbve_params& p, int threads = kThreads) {
-  const int w = threads == kThreads64Tiny ? kTileTXTiny : kTileTX;
+  const int w = threads <= kThreads64Small ? kTileTXTiny : kTileTX;
   return p.nx >= w ? w : p.nx;
 }
 
@@ -356,7 +359,7 @@ namespace {
 constexpr int kGraphSteps = 32;  // even, so a replay leaves the parity unchanged
 
 // Launch one time step of every tile list on stream st with the given parity.
-// With masks the step forks: the side stream runs the wall pass (which
+// With masks the step forks: the side stream runs the edge pass (which
 // completes the populations that wall nodes pull from solid nodes) and then
 // the masked tiles, while the plain tiles, which never read what the wall
 // pass writes, run on the caller's stream; the two join before the step ends.
@@ -369,14 +372,10 @@ int launch_one_step(lbve_handle* h, int parity, int flags, cudaStream_t st) {
     if (e != cudaSuccess) return cuda_fail(e, "fork of the masked-tile stream");
     for (int l = 0; l < kLists; ++l) {
       const int prec = l;
-      if (h->nmasked_inst[l] > 0 &&
-          launch_wall(prec, h->d_insts, h->d_walls[l], h->d_wrec[l], h->plan.wall_cap[l], parity,
-                      flags, h->side_stream))
-        return cuda_fail(cudaGetLastError(), "wall pass launch");
-      if (h->nopen_inst[l] > 0 &&
-          launch_column(prec, h->d_insts, h->d_cols[l], h->plan.ncols[l], parity,
-                        h->side_stream))
-        return cuda_fail(cudaGetLastError(), "column pass launch");
+      if (launch_edges(prec, h->d_insts, h->d_walls[l], h->d_wrec[l],
+                       h->nmasked_inst[l] > 0 ? h->plan.wall_cap[l] : 0, h->d_cols[l],
+                       h->nopen_inst[l] > 0 ? h->plan.ncols[l] : 0, parity, flags, h->side_stream))
+        return cuda_fail(cudaGetLastError(), "edge pass launch");
     }
   }
   for (int l = 0; l < kLists; ++l) {
@@ -448,6 +447,16 @@ void drop_graph(lbve_handle* h) {
 
 constexpr int kEx[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
 constexpr int kEy[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
+
+// Wall fraction of link d (1..8) of a wall node, and what the edge pass uses of it.
+void set_wall_fraction(WallDev& W, int d, double q) {
+  const bool below = q < 0.5;
+  const double r = 1.0 / (2.0 * q);
+  W.q[d - 1] = q;
+  W.a[d - 1] = below ? 2.0 * q : r;
+  W.b[d - 1] = below ? 1.0 - 2.0 * q : 1.0 - r;
+  W.fmask = (W.fmask & ~(1 << (16 + d))) | (below ? 1 << (16 + d) : 0);
+}
 
 // FNV-1a over the mask and the wall links: identifies the geometry a saved
 // state belongs to.
@@ -647,7 +656,7 @@ int install_mask(lbve_handle* h, int i, const uint8_t* mask) {
         W.k = (int32_t)k;
         W.umask = umask;
         W.fmask = fmask;
-        for (int d = 0; d < 8; ++d) W.q[d] = 0.5;
+        for (int d = 1; d < 9; ++d) set_wall_fraction(W, d, 0.5);
         index[k] = (int32_t)walls.size();
         walls.push_back(W);
       }
@@ -1366,7 +1375,7 @@ int lbve_set_wall_distances(lbve_handle* h, int32_t inst, int32_t n_links, const
                   node[j], dir[j]);
     if (!(q[j] > 0.0 && q[j] <= 1.0)) return set_error(LBVE_ERR_ARG, "link %d: q must be in (0, 1]", j);
   }
-  for (int32_t j = 0; j < n_links; ++j) W[idx[node[j]]].q[dir[j] - 1] = q[j];
+  for (int32_t j = 0; j < n_links; ++j) set_wall_fraction(W[idx[node[j]]], dir[j], q[j]);
   const cudaError_t e = upload_walls(h, inst);
   if (e != cudaSuccess) return cuda_fail(e, "wall upload");
   update_geometry_hash(h, inst);
@@ -1848,12 +1857,9 @@ extern "C" int lbve_adjoint_step_ex(lbve_handle* h, int32_t inst, const double* 
     }
     if ((ee = set_desc(src, state(to), hist_of(to))) != cudaSuccess)
       return cuda_fail(ee, "adjoint descriptor");
-    if (masked && !wcopy.empty() &&
-        launch_wall(prec, d_desc, d_walls, (double*)(ws + a.off_wrec), (int)wcopy.size(), 0, 0,
-                    st))
-      return cuda_fail(cudaGetLastError(), "adjoint wall pass");
-    if (open && launch_column(prec, d_desc, (const ColTask*)(ws + a.off_cols), 2 * p.ny, 0, st))
-      return cuda_fail(cudaGetLastError(), "adjoint column pass");
+    if (launch_edges(prec, d_desc, d_walls, (double*)(ws + a.off_wrec), (int)wcopy.size(),
+                     (const ColTask*)(ws + a.off_cols), open ? 2 * p.ny : 0, 0, 0, st))
+      return cuda_fail(cudaGetLastError(), "adjoint edge pass");
     if (!launch_tiles(kModeStep, 0)) return cuda_fail(cudaGetLastError(), "adjoint forward step");
     return LBVE_OK;
   };

@@ -14,7 +14,7 @@ int set_error(int code, const char* fmt, ...) __attribute__((format(printf, 2, 3
 // SM give 21 warps in seven independent load / barrier / compute phases.
 // Float64 (bound by the FP64 pipe): 256 (32 x 8 tiles), two per SM.  A
 // float64 batch too small to give every SM one such tile runs 64-thread CTAs
-// (32 x 2 tiles, eight per SM, the same registers per thread) instead: each
+// (8 x 8 tiles) instead: each
 // SM's FP64 pipe then has a quarter of the nodes to work through.
 #ifndef LBVE_THREADS
 #define LBVE_THREADS 96
@@ -38,7 +38,7 @@ constexpr int kThreads = LBVE_THREADS;          // float32 step kernel
 constexpr int kThreads64 = LBVE_THREADS_FP64;   // float64 step kernel
 constexpr int kThreads64Small = LBVE_THREADS_FP64_SMALL;  // float64, small batches
 constexpr int kThreads64Tiny = LBVE_THREADS_FP64_TINY;    // float64, tiny batches
-constexpr int kTileTXTiny = 8;  // default tile width of the one-warp float64 CTAs
+constexpr int kTileTXTiny = 8;  // default tile width of the one- and two-warp float64 CTAs
 constexpr int kNumSMs = 152;  // GB300; sizes the small-batch choice only
 constexpr int kTileTX = LBVE_TILE_TX;   // default tile width (nodes along x) for nx >= kTileTX
 // threads per CTA (for float64, the size of all but small batches) and the
@@ -141,16 +141,19 @@ struct alignas(16) TileDev {
 // One fluid node next to the solid mask (the compact link list of the wall
 // pass).  inst < 0 marks an unused record.
 //   umask bit i: link i is a wall link (node k - e_i is solid)
-//   fmask bit i: node k + e_i is fluid (second operand of the interpolation)
+//   fmask bit i: node k + e_i is fluid (second operand of the interpolation);
+//         bit 16 + i: q of link i is below 1/2
 //   q[i-1]:      wall fraction of link i, in (0, 1]
-struct WallDev {
+//   a, b[i-1]:   weights of the interpolation's operands: 2q, 1 - 2q below 1/2,
+//                else 1/(2q), 1 - 1/(2q)
+struct alignas(16) WallDev {
   int32_t inst, k, umask, fmask;
-  double q[8];
+  double q[8], a[8], b[8];
 };
 constexpr int kWallRec = 8;  // drag x, drag y, wall in x3, wall out x3
 
 // One node of an open column: {instance, row, side (0 inlet, 1 outlet)}.
-struct ColTask {
+struct alignas(16) ColTask {
   int32_t inst, y, side, pad;
 };
 
@@ -163,15 +166,13 @@ enum : int { kModeStep = 0, kModeInit = 1 };
 int launch_step(int prec, int threads, const InstDev* d_insts, const TileDev* d_tiles,
                 int n_tiles, int parity, int mode, int flags, double* d_partials, void* stream,
                 int masked = 0);
-// Wall pass before a step: completes the populations of the wall links of
-// n_walls records in the buffer pop[parity]; on the final step it writes one
-// kWallRec record per wall node to d_rec (lbve_wall.cu).
-int launch_wall(int prec, const InstDev* d_insts, const WallDev* d_walls, double* d_rec,
-                int n_walls, int parity, int flags, void* stream);
-// Column pass before a step: the completed populations of the open columns'
-// nodes (n_tasks of them) into each instance's colbuf (lbve_wall.cu).
-int launch_column(int prec, const InstDev* d_insts, const ColTask* d_tasks, int n_tasks,
-                  int parity, void* stream);
+// Edge pass before a step (lbve_wall.cu): completes the populations of the wall
+// links of n_walls records in the buffer pop[parity], on the final step with
+// one kWallRec record per wall node in d_rec, and the populations of n_tasks
+// open-column nodes in their instances' colbuf.
+int launch_edges(int prec, const InstDev* d_insts, const WallDev* d_walls, double* d_rec,
+                 int n_walls, const ColTask* d_tasks, int n_tasks, int parity, int flags,
+                 void* stream);
 // Adjoint pass modes: a normal step, the final fields (the loss), the initial collision.
 enum : int { kAdjStep = 0, kAdjFields = 1, kAdjInit = 2 };
 

@@ -43,10 +43,14 @@ static int launch_step_t(const InstDev* d_insts, const TileDev* d_tiles, int n_t
   return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;  // the caller reads and clears it
 }
 
-template <typename R, int NT>
+// Masked tiles take more threads than nodes, so that other warps than those of
+// the nodes cover the halo ring, in one round (134 ring nodes of a 32 x 3
+// float32 tile, 48 of an 8 x 8 float64 one; wider rings loop): there are few such
+// tiles, and each is a serial chain (float32 10.8 -> 8.6 us, isolated).
+template <typename R, int NT, int NTM>
 static int launch_step_m(const InstDev* d_insts, const TileDev* d_tiles, int n_tiles, int parity,
                          int mode, int flags, double* d_partials, cudaStream_t st, int masked) {
-  return masked ? launch_step_t<R, true, NT>(d_insts, d_tiles, n_tiles, parity, mode, flags,
+  return masked ? launch_step_t<R, true, NTM>(d_insts, d_tiles, n_tiles, parity, mode, flags,
                                              d_partials, st)
                 : launch_step_t<R, false, NT>(d_insts, d_tiles, n_tiles, parity, mode, flags,
                                               d_partials, st);
@@ -58,7 +62,7 @@ int launch_step(int prec, int threads, const InstDev* d_insts, const TileDev* d_
                 int masked) {
   cudaStream_t st = (cudaStream_t)stream;
   if (prec == 0 && threads == kThreads64)
-    return launch_step_m<double, kThreads64>(d_insts, d_tiles, n_tiles, parity, mode, flags,
+    return launch_step_m<double, kThreads64, kThreads64>(d_insts, d_tiles, n_tiles, parity, mode, flags,
                                              d_partials, st, masked);
   if (prec == 0 && threads == kThreads64Tiny) {
     // tiles of at most 32 nodes: the time steps of plain tiles spread each
@@ -72,14 +76,14 @@ int launch_step(int prec, int threads, const InstDev* d_insts, const TileDev* d_
                                                                     d_partials);
       return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;  // the caller reads and clears it
     }
-    return launch_step_m<double, kThreads64Tiny>(d_insts, d_tiles, n_tiles, parity, mode, flags,
+    return launch_step_m<double, kThreads64Tiny, 64>(d_insts, d_tiles, n_tiles, parity, mode, flags,
                                                  d_partials, st, masked);
   }
   if (prec == 0 && threads == kThreads64Small)
-    return launch_step_m<double, kThreads64Small>(d_insts, d_tiles, n_tiles, parity, mode, flags,
+    return launch_step_m<double, kThreads64Small, 128>(d_insts, d_tiles, n_tiles, parity, mode, flags,
                                                   d_partials, st, masked);
   if (prec == 1 && threads == kThreads)
-    return launch_step_m<float, kThreads>(d_insts, d_tiles, n_tiles, parity, mode, flags,
+    return launch_step_m<float, kThreads, 160>(d_insts, d_tiles, n_tiles, parity, mode, flags,
                                           d_partials, st, masked);
   if (prec == 2 && threads == kThreads && !masked)  // float32 pairs: plain tiles only
     return launch_step_t<df32, false, kThreads>(d_insts, d_tiles, n_tiles, parity, mode, flags,

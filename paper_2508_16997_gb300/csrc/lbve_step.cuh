@@ -1013,10 +1013,10 @@ __device__ __forceinline__ void collide_node(const InstDev& D, int k, int S, R* 
 // Resident CTAs per SM the register budget is sized for: the float32 step
 // is HBM-bound and wants more loads in flight; the float64 step is bound by
 // the FP64 pipe.
-// Masked tiles carry the mask's one-sided differences: a budget of 5 CTAs
-// per SM lets them keep their registers without spills.
+// Masked tiles carry the mask's one-sided differences: a budget of 3 CTAs of
+// 160 threads per SM lets them keep their registers without spills.
 #ifndef LBVE_FP32_MASKED_MIN_BLOCKS
-#define LBVE_FP32_MASKED_MIN_BLOCKS 5
+#define LBVE_FP32_MASKED_MIN_BLOCKS 3
 #endif
 // Float64 CTAs: 256 threads two per SM (128 registers per thread).  The
 // 64- and one-warp CTAs serve batches with fewer tiles than 4 and 2 per SM,
@@ -1032,7 +1032,7 @@ struct MinBlocks {
       std::is_same<R, df32>::value
           ? LBVE_DF32_MIN_BLOCKS
           : sizeof(R) == 4 ? (MASKED ? LBVE_FP32_MASKED_MIN_BLOCKS : LBVE_FP32_MIN_BLOCKS)
-                           : (NT <= 32 ? 2 : NT <= 64 ? 4 : (NT <= 512 ? 512 / NT : 1));
+                           : (NT <= 32 ? 2 : NT <= 64 ? 4 : MASKED && NT < 256 ? 1 : 512 / NT);
 };
 
 // Open channels: nodes of the inlet (x = 0) and outlet (x = nx - 1) columns
@@ -1265,12 +1265,33 @@ __device__ __forceinline__ void process_tile(const InstDev* __restrict__ insts, 
   const int x = T.x0 + tx, y = T.y0 + ty;
   const bool inside = in_tile && (x < nx) && (y < ny);
   // solid-mask nodes (masked tiles only) take no part in the update
-  const bool solid = MASKED && inside && D.mask && D.mask[y * nx + x] != 0;
-  const bool active = inside && !solid;
+  // (rows 0..2 and ny-3.. of a walled domain and the three columns at open ends
+  // carry no mask, so what follows here may look at the position alone and
+  // the loads below need not wait for the mask); sxp..sym: blocked sides
+  bool solid = false, sxp = false, sxm = false, syp = false, sym = false;
   const int ri = (ty + hy) * RW + tx + 1;  // this slot in the halo region
-  const bool wb = active && !py && y == 0, wt = active && !py && y == ny - 1;
+  const bool wb = inside && !py && y == 0, wt = inside && !py && y == ny - 1;
   // an open column's node arrives completed (colbuf): no wall completion there
-  const bool ocol = MASKED && MODE == kModeStep && active && open_column(D, x);
+  const bool ocol = MASKED && MODE == kModeStep && inside && open_column(D, x);
+  if (MASKED && inside) {
+    // a side is blocked by a solid node or, in an open channel, by the end of
+    // the domain beyond the inlet / outlet column
+    sxp = D.open_x && x == nx - 1;
+    sxm = D.open_x && x == 0;
+    if (const uint8_t* __restrict__ M = D.mask) {
+      const int xp = x == nx - 1 ? 0 : x + 1, xm = x == 0 ? nx - 1 : x - 1;
+      const int yp = y == ny - 1 ? (py ? 0 : y) : y + 1, ym = y == 0 ? (py ? ny - 1 : y) : y - 1;
+      const uint8_t m0 = M[y * nx + x], m1 = M[y * nx + xp], m2 = M[y * nx + xm];
+      const uint8_t m3 = M[yp * nx + x], m4 = M[ym * nx + x];
+      solid = m0 != 0;
+      sxp = sxp || m1 != 0;
+      sxm = sxm || m2 != 0;
+      // rows next to a flat wall carry no mask, so y +- 1 lies in the domain
+      syp = !wb && !wt && m3 != 0;
+      sym = !wb && !wt && m4 != 0;
+    }
+  }
+  const bool active = inside && !solid;
   const bool wcomp = (wb || wt) && !ocol;
   const int nring = 2 * hy * TX + 2 * TY;  // the halo ring without its corners
 
@@ -1308,7 +1329,7 @@ __device__ __forceinline__ void process_tile(const InstDev* __restrict__ insts, 
   R d[9], g[3][9], So[3] = {R(0), R(0), R(0)}, uxo = R(0), uyo = R(0), Fx = Fx0, Fy = Fy0;
   R post[3][3];  // own outgoing-to-wall post-collision slots (wall rows only)
   int k = 0;
-  if (active) {
+  if (inside) {
     k = y * nx + x;
     int rm, rp;
     neighbour_rows(y, nx, ny, py, rm, rp);
@@ -1428,12 +1449,7 @@ __device__ __forceinline__ void process_tile(const InstDev* __restrict__ insts, 
     if constexpr (MASKED) {
       // one-sided differences where an axis neighbour is solid; the values
       // two nodes away come straight from the pulled populations (L2)
-      // a side is blocked by a solid node or, in an open channel, by the
-      // end of the domain beyond the inlet / outlet column
       const uint8_t* __restrict__ M = D.mask;
-      const int xp = x == nx - 1 ? 0 : x + 1, xm = x == 0 ? nx - 1 : x - 1;
-      const bool sxp = (D.open_x && x == nx - 1) || (M && M[y * nx + xp] != 0);
-      const bool sxm = (D.open_x && x == 0) || (M && M[y * nx + xm] != 0);
       if (sxp || sxm) {
         if (sxp && sxm) {
           Arith<R>::blocked(0, G);
@@ -1449,25 +1465,20 @@ __device__ __forceinline__ void process_tile(const InstDev* __restrict__ insts, 
           Arith<R>::one_sided(0, t, Q, ri, i1, f, has2, w, G);
         }
       }
-      if (!wb && !wt && M) {
-        // rows next to a flat wall carry no mask, so y +- 1 lies in the domain
-        const int yp = (py && y == ny - 1) ? 0 : y + 1, ym = (py && y == 0) ? ny - 1 : y - 1;
-        const bool syp = M[yp * nx + x] != 0, sym = M[ym * nx + x] != 0;
-        if (syp || sym) {
-          if (syp && sym) {
-            Arith<R>::blocked(1, G);
-          } else {
-            const int t = syp ? -1 : 1;
-            const int i1 = t > 0 ? ri + RW : ri - RW;
-            int y2 = y + 2 * t;
-            if (py) y2 = ((y2 % ny) + ny) % ny;
-            const bool has2 = y2 >= 0 && y2 < ny && M[y2 * nx + x] == 0;
-            Flow<R> w;
-            w.rest();
-            if (has2)
-              region_flow<R, MODE>(D, src, force, ffield, Fx0, Fy0, S, nx, ny, py, x, y2, w);
-            Arith<R>::one_sided(1, t, Q, ri, i1, f, has2, w, G);
-          }
+      if (syp || sym) {
+        if (syp && sym) {
+          Arith<R>::blocked(1, G);
+        } else {
+          const int t = syp ? -1 : 1;
+          const int i1 = t > 0 ? ri + RW : ri - RW;
+          int y2 = y + 2 * t;
+          if (py) y2 = ((y2 % ny) + ny) % ny;
+          const bool has2 = y2 >= 0 && y2 < ny && M[y2 * nx + x] == 0;
+          Flow<R> w;
+          w.rest();
+          if (has2)
+            region_flow<R, MODE>(D, src, force, ffield, Fx0, Fy0, S, nx, ny, py, x, y2, w);
+          Arith<R>::one_sided(1, t, Q, ri, i1, f, has2, w, G);
         }
       }
     }
