@@ -18,7 +18,8 @@
 //               adjoints of rho and u; writes lambda_t's history part
 //   adj_gather  transposed gradient stencils + u/rho chain + Zou-He reverse;
 //               writes lambda of the hydro pulls, accumulates dL/dF
-//   adj_pull    reverse pull into lambda_t's populations
+//   adj_pull    reverse pull into lambda_t's populations (masks and open columns
+//               only: else the first two passes write lambda_t themselves)
 // A fourth kernel (adj_moments) recomputes rho, u of the forward state so the
 // gather can read its neighbours.  Open channels add a fifth between the
 // gather and the pull (adj_column): the inlet and outlet nodes' completed
@@ -506,10 +507,36 @@ __device__ __forceinline__ void cnebb_mask_T(const R gp[9], const R pm[9], R del
   }
 }
 
+// Reverse pull without a mask or open columns, from the pulling side: lambda of
+// the pulled population i of node (x, y) is lambda_t's at the node it came from,
+// (x, y) - e_i.  An unknown direction of a flat-wall row came from nowhere; its
+// entry is lambda of the node's own population in the opposite direction (zero
+// for the hydrodynamic lattice).  Each entry of lambda_t is written once, and
+// the separate pass over 36 values per node (26 us of 120 per reversed step on
+// a 512^2 grid) falls away.
+template <typename R>
+__device__ __forceinline__ void push_lambda(const InstDev& D, R* __restrict__ lam, int x, int y,
+                                            const R ld[9]) {
+  const int nx = D.nx, ny = D.ny, S = D.stride, k = y * nx + x;
+  const int xm = x == 0 ? nx - 1 : x - 1, xp = x == nx - 1 ? 0 : x + 1;
+  const bool py = D.periodic_y != 0;
+  const int rm = y > 0 ? k - x - nx : (py ? (ny - 1) * nx : -1);      // row y - 1
+  const int rp = y < ny - 1 ? k - x + nx : (py ? 0 : -1);             // row y + 1
+  lam[k] = ld[0];
+  lam[(size_t)1 * S + k - x + xm] = ld[1];
+  lam[(size_t)3 * S + k - x + xp] = ld[3];
+  lam[(size_t)(rm >= 0 ? 2 : 4) * S + (rm >= 0 ? rm + x : k)] = ld[2];
+  lam[(size_t)(rm >= 0 ? 5 : 7) * S + (rm >= 0 ? rm + xm : k)] = ld[5];
+  lam[(size_t)(rm >= 0 ? 6 : 8) * S + (rm >= 0 ? rm + xp : k)] = ld[6];
+  lam[(size_t)(rp >= 0 ? 4 : 2) * S + (rp >= 0 ? rp + x : k)] = ld[4];
+  lam[(size_t)(rp >= 0 ? 7 : 5) * S + (rp >= 0 ? rp + xp : k)] = ld[7];
+  lam[(size_t)(rp >= 0 ? 8 : 6) * S + (rp >= 0 ? rp + xm : k)] = ld[8];
+}
+
 // Pass 1: local reverse of the collision, source, history and CNEBB.
 // float32: a budget of 128 registers (two CTAs per SM) trades a few spills
 // for twice the warps in flight; float64 keeps its full register file.
-template <typename R, int MODE, bool OPEN>
+template <typename R, int MODE, bool OPEN, bool PUSH>
 __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1)
     adj_local(const InstDev* __restrict__ Dp, AdjArgs<R> A) {
   const InstDev& D = *Dp;
@@ -843,9 +870,13 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1)
 #pragma unroll
         for (int i = 0; i < 9; ++i) ld[i] = lg[i];
       }
-      R* lp = A.lam_pulled + (size_t)(9 + 9 * l) * S + k;
+      if (PUSH) {
+        push_lambda<R>(D, A.lam_cur + (size_t)(9 + 9 * l) * S, x, y, ld);
+      } else {
+        R* lp = A.lam_pulled + (size_t)(9 + 9 * l) * S + k;
 #pragma unroll
-      for (int i = 0; i < 9; ++i) lp[(size_t)i * S] = ld[i];
+        for (int i = 0; i < 9; ++i) lp[(size_t)i * S] = ld[i];
+      }
     }
   }
   A.lam_G[k] = lG[0];
@@ -866,7 +897,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1)
 // Pass 2: gather the transposed gradient stencils, reverse u = (j + F/2)/rho
 // and the hydro moments, reverse Zou-He; writes lambda of the hydro pulls and
 // accumulates dL/dF.
-template <typename R, int MODE, bool OPEN>
+template <typename R, int MODE, bool OPEN, bool PUSH>
 __global__ void adj_gather(const InstDev* __restrict__ Dp, AdjArgs<R> A) {
   const InstDev& D = *Dp;
   const int nx = D.nx, ny = D.ny, S = D.stride, n = nx * ny;
@@ -954,8 +985,12 @@ __global__ void adj_gather(const InstDev* __restrict__ Dp, AdjArgs<R> A) {
       for (int i = 1; i < 9; ++i)
         if ((um >> i) & 1) ld[i] -= (R)(A.drag_w[0] * aex(i) + A.drag_w[1] * aey(i));
     }
+    if (PUSH) {
+      push_lambda<R>(D, A.lam_cur, x, y, ld);
+    } else {
 #pragma unroll
-    for (int i = 0; i < 9; ++i) A.lam_pulled[(size_t)i * S + k] = ld[i];
+      for (int i = 0; i < 9; ++i) A.lam_pulled[(size_t)i * S + k] = ld[i];
+    }
   }
   A.dF[k] += (double)lFx;
   A.dF[n + k] += (double)lFy;

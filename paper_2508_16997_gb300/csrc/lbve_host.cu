@@ -764,7 +764,7 @@ int lbve_create(const lbve_params* p, int32_t n, void* d_workspace, size_t bytes
     std::memset(&D, 0, sizeof(D));
     D.pop[0] = h->ws + q.off_pop[0];
     D.pop[1] = h->ws + q.off_pop[1];
-    D.hist = h->ws + q.off_hist;
+    D.hist = D.hist_out = h->ws + q.off_hist;
     D.force = h->ws + q.off_force;
     D.fields = (double*)(h->ws + q.off_fields);
     D.nx = p[i].nx;
@@ -1615,6 +1615,16 @@ struct AdjPlan {
   int nwall, nmtiles;
   size_t off_scratch, off_walls, off_wrec, off_widx, off_mtiles;
   size_t off_cols;  // open channels: the column tasks of the instance (2 ny)
+  // Descriptors, one per kind of step, uploaded once: each names the state it
+  // reads and the one it writes.  (Uploaded before each step, with a device copy
+  // of the history, they took 15 % of a reversed step on a 512^2 grid.)
+  size_t desc_init() const { return 0; }                      // staged fields -> checkpoint 0
+  size_t desc_roll(int64_t m) const { return 1 + m; }         // segment state m % 2 -> (m + 1) % 2
+  size_t desc_leave(int64_t j) const { return 3 + j; }        // checkpoint j -> segment 0 (or j + 1)
+  size_t desc_enter(int64_t j) const { return 3 + nck + j; }  // last rolling state -> checkpoint j
+  size_t desc_seg(int64_t m) const { return 3 + 2 * nck + m; }        // segment state m -> m + 1
+  size_t desc_rev(int64_t m) const { return 3 + 2 * nck + s + m; }    // reverse of segment state m
+  size_t ndesc() const { return 3 + 2 * nck + 2 * s + 2; }
 };
 
 // The square-root checkpoint interval: ceil(sqrt(T)).
@@ -1643,7 +1653,7 @@ AdjPlan make_adj_plan(const lbve_params& p, const InstPlan& q, int64_t T, int nw
     off = align_up(off + std::max<size_t>(bytes, 1), kAlign);
     return o;
   };
-  a.off_desc = take(sizeof(InstDev));
+  a.off_desc = take(sizeof(InstDev) * a.ndesc());
   a.off_tiles = take(sizeof(TileDev) * q.ntiles);
   a.off_partials = take(sizeof(double) * kPartial * q.ntiles);
   a.off_fields = take(sizeof(double) * 6 * q.stride);
@@ -1806,24 +1816,15 @@ extern "C" int lbve_adjoint_step_ex(lbve_handle* h, int32_t inst, const double* 
     if (e != cudaSuccess) return cuda_fail(e, "adjoint mask tables");
   }
   const int nmt = (int)mtiles.size();
-  auto launch_tiles = [&](int mode, int flags) -> bool {
+  auto launch_tiles = [&](size_t at, int mode, int flags) -> bool {
     const int nt = h->plan.threads[q.list];
-    if (launch_step(prec, nt, d_desc, d_tiles, q.ntiles, 0, mode, flags, d_partials, st))
+    if (launch_step(prec, nt, d_desc + at, d_tiles, q.ntiles, 0, mode, flags, d_partials, st))
       return false;
     if (nmt > 0 &&
-        launch_step(prec, nt, d_desc, d_mtiles, nmt, 0, mode, flags, d_partials, st, 1))
+        launch_step(prec, nt, d_desc + at, d_mtiles, nmt, 0, mode, flags, d_partials, st, 1))
       return false;
     return true;
   };
-  auto set_desc = [&](void* pop0, void* pop1, void* hist) -> cudaError_t {
-    D.pop[0] = pop0;
-    D.pop[1] = pop1;
-    D.hist = hist;
-    // ordered on the stream; a pageable source is staged before the call
-    // returns, so D may change right after
-    return cudaMemcpyAsync(d_desc, &D, sizeof(InstDev), cudaMemcpyHostToDevice, st);
-  };
-  auto state = [&](char* base) { return base; };
   auto hist_of = [&](char* st_) { return st_ + 36 * plane; };
   char* ck = ws + a.off_ck;
   char* seg = ws + a.off_seg;
@@ -1840,43 +1841,64 @@ extern "C" int lbve_adjoint_step_ex(lbve_handle* h, int32_t inst, const double* 
                           st);
   }
   if (e != cudaSuccess) return cuda_fail(e, "adjoint initial-field upload");
-  if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_fail(e, "adjoint set-up");
+  // the descriptors of every step; with a mask the wall pass completes a scratch
+  // copy of the state read, so stored states stay raw (the reverse passes redo
+  // the completion)
+  auto ckp = [&](int64_t j) { return ck + j * a.state_bytes; };
+  auto segp = [&](int64_t m) { return seg + m * a.state_bytes; };
+  std::vector<InstDev> descs(a.ndesc(), D);
+  auto put_desc = [&](size_t at, char* from, char* to) {
+    InstDev& E = descs[at];
+    E.pop[0] = masked ? scratch : from;
+    E.pop[1] = to;
+    E.hist = hist_of(from);
+    E.hist_out = hist_of(to);
+  };
+  {
+    InstDev& E = descs[a.desc_init()];
+    E.pop[0] = stage;
+    E.pop[1] = ck;
+    E.hist = E.hist_out = hist_of(ck);
+  }
+  for (int64_t m = 0; m < 2; ++m)
+    if (a.s > 1) put_desc(a.desc_roll(m), segp(m), segp(1 - m));
+  for (int64_t j = 0; j < a.nck; ++j) {
+    put_desc(a.desc_leave(j), ckp(j), a.s > 1 ? segp(0) : ckp(std::min(j + 1, a.nck - 1)));
+    if (a.s > 1) put_desc(a.desc_enter(j), segp((a.s - 2) % 2), ckp(j));
+  }
+  for (int64_t m = 0; m + 1 < a.s; ++m) put_desc(a.desc_seg(m), segp(m), segp(m + 1));
+  // the reverse passes take sizes, coefficients and flags from theirs; the state
+  // comes with their arguments
+  for (int64_t m = 0; m < a.s; ++m) put_desc(a.desc_rev(m), segp(m), segp(m));
+  e = cudaMemcpyAsync(d_desc, descs.data(), sizeof(InstDev) * descs.size(), cudaMemcpyHostToDevice,
+                      st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) return cuda_fail(e, "adjoint set-up");
 
-  // one forward step from state `from` into state `to` (history copied, then
-  // updated in place).  With a mask the wall pass completes a scratch copy of
-  // `from`, so stored states stay raw (the reverse passes redo the completion).
-  auto fwd = [&](char* from, char* to) -> int {
-    cudaError_t ee = cudaMemcpyAsync(hist_of(to), hist_of(from), 5 * plane,
-                                     cudaMemcpyDeviceToDevice, st);
-    if (ee != cudaSuccess) return cuda_fail(ee, "adjoint history copy");
-    char* src = state(from);
+  // one forward step of the descriptor `at`, whose state read is `from`
+  auto fwd = [&](size_t at, char* from) -> int {
     if (masked) {
-      ee = cudaMemcpyAsync(scratch, state(from), 36 * plane, cudaMemcpyDeviceToDevice, st);
+      const cudaError_t ee = cudaMemcpyAsync(scratch, from, 36 * plane, cudaMemcpyDeviceToDevice,
+                                             st);
       if (ee != cudaSuccess) return cuda_fail(ee, "adjoint scratch copy");
-      src = scratch;
     }
-    if ((ee = set_desc(src, state(to), hist_of(to))) != cudaSuccess)
-      return cuda_fail(ee, "adjoint descriptor");
-    if (launch_edges(prec, d_desc, d_walls, (double*)(ws + a.off_wrec), (int)wcopy.size(),
+    if (launch_edges(prec, d_desc + at, d_walls, (double*)(ws + a.off_wrec), (int)wcopy.size(),
                      (const ColTask*)(ws + a.off_cols), open ? 2 * p.ny : 0, 0, 0, st))
       return cuda_fail(cudaGetLastError(), "adjoint edge pass");
-    if (!launch_tiles(kModeStep, 0)) return cuda_fail(cudaGetLastError(), "adjoint forward step");
+    if (!launch_tiles(at, kModeStep, 0))
+      return cuda_fail(cudaGetLastError(), "adjoint forward step");
     return LBVE_OK;
   };
 
   // ---- forward sweep: X_0 from the initial fields, checkpoints every s steps ----
-  if ((e = set_desc(stage, state(ck), hist_of(ck))) != cudaSuccess)
-    return cuda_fail(e, "adjoint descriptor");
-  if (!launch_tiles(kModeInit, kFinal)) return cuda_fail(cudaGetLastError(), "adjoint init step");
+  if (!launch_tiles(a.desc_init(), kModeInit, kFinal))
+    return cuda_fail(cudaGetLastError(), "adjoint init step");
   for (int64_t j = 1; j < a.nck; ++j) {
     // X_{j s} from X_{(j-1) s}: s steps through two rolling buffers of the segment area
-    char* cur = ck + (j - 1) * a.state_bytes;
-    for (int64_t m = 0; m < a.s; ++m) {
-      char* nxt = (m == a.s - 1) ? ck + j * a.state_bytes : seg + (m % 2) * a.state_bytes;
-      const int rc = fwd(cur, nxt);
-      if (rc) return rc;
-      cur = nxt;
-    }
+    int rc = fwd(a.desc_leave(j - 1), ckp(j - 1));
+    for (int64_t m = 1; m < a.s && !rc; ++m)
+      rc = fwd(m == a.s - 1 ? a.desc_enter(j) : a.desc_roll((m - 1) % 2), segp((m - 1) % 2));
+    if (rc) return rc;
   }
 
   // ---- reverse sweep ----
@@ -1907,6 +1929,7 @@ extern "C" int lbve_adjoint_step_ex(lbve_handle* h, int32_t inst, const double* 
     A.drag_w[1] = dL_ddrag[1];
   }
   A.open = open ? 1 : 0;
+  A.push = !open && !masked;
   // without a field loss the final pass reads zeros
   const double* fields_seed = d_dL_dfields;
   if (!fields_seed) {
@@ -1917,8 +1940,8 @@ extern "C" int lbve_adjoint_step_ex(lbve_handle* h, int32_t inst, const double* 
   char* lam[2] = {ws + a.off_lam[0], ws + a.off_lam[1]};
   int li = 0;  // lam[li] holds lambda of the most recent (later) state
   const int n_nodes = (int)nn;
-  auto pass = [&](int mode, int which) -> int {
-    if (launch_adjoint(prec, mode, which, d_desc, A, n_nodes, st))
+  auto pass = [&](size_t at, int mode, int which) -> int {
+    if (launch_adjoint(prec, mode, which, d_desc + at, A, n_nodes, st))
       return cuda_fail(cudaGetLastError(), "adjoint pass launch");
     return LBVE_OK;
   };
@@ -1933,13 +1956,12 @@ extern "C" int lbve_adjoint_step_ex(lbve_handle* h, int32_t inst, const double* 
       if (e != cudaSuccess) return cuda_fail(e, "adjoint checkpoint copy");
     }
     for (int64_t m = m0 + 1; m < m1; ++m) {
-      const int rc = fwd(seg + (m - 1 - m0) * a.state_bytes, seg + (m - m0) * a.state_bytes);
+      const int rc = fwd(a.desc_seg(m - 1 - m0), segp(m - 1 - m0));
       if (rc) return rc;
     }
     for (int64_t m = m1 - 1; m >= m0; --m) {
-      char* X = a.s > 1 ? seg + (m - m0) * a.state_bytes : ck + j * a.state_bytes;
-      if ((e = set_desc(state(X), state(X), hist_of(X))) != cudaSuccess)
-        return cuda_fail(e, "adjoint descriptor");
+      char* X = a.s > 1 ? segp(m - m0) : ckp(j);
+      const size_t at = a.desc_rev(m - m0);
       A.X = X;
       A.lam_cur = lam[li ^ 1];
       int mode;
@@ -1955,27 +1977,25 @@ extern "C" int lbve_adjoint_step_ex(lbve_handle* h, int32_t inst, const double* 
         A.lam_fields = nullptr;
         A.final_pass = 0;
       }
-      int rc = pass(mode, 0);
-      if (!rc) rc = pass(mode, 1);
-      if (!rc) rc = pass(mode, 2);
-      if (!rc && open && launch_adjoint(prec, mode, 4, d_desc, A, 2 * p.ny, st))
+      int rc = pass(at, mode, 0);
+      if (!rc) rc = pass(at, mode, 1);
+      if (!rc) rc = pass(at, mode, 2);
+      if (!rc && open && launch_adjoint(prec, mode, 4, d_desc + at, A, 2 * p.ny, st))
         rc = cuda_fail(cudaGetLastError(), "adjoint column reverse launch");
-      if (!rc) rc = pass(mode, 3);
+      if (!rc && !A.push) rc = pass(at, mode, 3);
       if (rc) return rc;
       li ^= 1;
     }
   }
   // the initial collision (X_0 from the equilibrium of the initial fields)
-  if ((e = set_desc(stage, ck, hist_of(ck))) != cudaSuccess)
-    return cuda_fail(e, "adjoint descriptor");
   A.X = nullptr;
   A.lam_next = lam[li];
   A.lam_fields = nullptr;
   A.lam_cur = lam[li ^ 1];
   A.final_pass = 0;
-  int rc = pass(kAdjInit, 0);
-  if (!rc) rc = pass(kAdjInit, 1);
-  if (!rc) rc = pass(kAdjInit, 2);
+  int rc = pass(a.desc_init(), kAdjInit, 0);
+  if (!rc) rc = pass(a.desc_init(), kAdjInit, 1);
+  if (!rc) rc = pass(a.desc_init(), kAdjInit, 2);
   if (rc) return rc;
   if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return cuda_fail(e, "lbve_adjoint_step");
   return LBVE_OK;

@@ -123,6 +123,9 @@ struct alignas(16) InstDev {
                                  // columns (inlet rows, then outlet rows), deviations
   const double* inlet;           // [5][ny] u_x, u_y, A_xx, A_xy, A_yy at the inlet
   double inv_Uc;
+  void* hist_out;      // [5][stride]  history that a step writes: hist, or the next
+                       // state's where states are kept (adjoint)
+  double pad;
   double cd[20];
   float cl[20];
 };
@@ -200,6 +203,8 @@ struct AdjArgsRaw {
   double drag_w[2];
   int final_pass;
   int open;  // open channel: the node passes are the variants with the open columns
+  int push;  // no mask, no open column: the local and gather passes write lam_cur, there is
+             // no reverse pull
 };
 // pass: 0 moments, 1 local reverse, 2 gather, 3 reverse pull, 4 reverse of an
 // open channel's column pass (n_nodes = 2 ny: one thread per open-column

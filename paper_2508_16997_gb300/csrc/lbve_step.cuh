@@ -1238,7 +1238,7 @@ __device__ __forceinline__ void process_tile(const InstDev* __restrict__ insts, 
   const R* __restrict__ srcR = (const R*)src;
   R* __restrict__ dst = (R*)D.pop[parity ^ 1];
   const R* __restrict__ force = (const R*)D.force;
-  R* __restrict__ hist = (R*)D.hist;
+  const R* hist = (const R*)D.hist;
   const bool ffield = D.force_field != 0;
   const R Fx0 = coef<R>(D, kCoefFx), Fy0 = coef<R>(D, kCoefFy);
   const int RW = TX + 2;
@@ -1504,8 +1504,8 @@ __device__ __forceinline__ void process_tile(const InstDev* __restrict__ insts, 
       ux_prev = (PartT<R>)__ldcg(D.fields + S + k);
       uy_prev = (PartT<R>)__ldcg(D.fields + 2 * S + k);
     }
-    collide_node<R, MODE, FINAL, MASKED>(D, k, S, dst, hist, hm, cm, f, G, Fx, Fy, So[0], So[1],
-                                         So[2], uxo, uyo, ux_prev, uy_prev, part, plo);
+    collide_node<R, MODE, FINAL, MASKED>(D, k, S, dst, (R*)D.hist_out, hm, cm, f, G, Fx, Fy, So[0],
+                                         So[1], So[2], uxo, uyo, ux_prev, uy_prev, part, plo);
   } else if (FINAL && solid) {
     // a solid node reports zero fields and adds nothing to the totals
     const int ks = y * nx + x;
@@ -1572,7 +1572,7 @@ __device__ __forceinline__ void process_tile_split(const InstDev* __restrict__ i
   const R* __restrict__ srcR = (const R*)src;
   R* __restrict__ dst = (R*)D.pop[parity ^ 1];
   const R* __restrict__ force = (const R*)D.force;
-  R* __restrict__ hist = (R*)D.hist;
+  const R* hist = (const R*)D.hist;
   const bool ffield = D.force_field != 0;
   const R Fx0 = coef<R>(D, kCoefFx), Fy0 = coef<R>(D, kCoefFy);
   const int RW = TX + 2;
@@ -1712,15 +1712,16 @@ __device__ __forceinline__ void process_tile_split(const InstDev* __restrict__ i
         uy_prev = D.fields[2 * S + k];
       }
       collide_hydro<R>(D, k, S, dst, hm, f, G, Fxx, Fxy, Fyy, Fx, Fy);
-      hist[3 * S + k] = f.ux;
-      hist[4 * S + k] = f.uy;
+      R* hist_out = (R*)D.hist_out;
+      hist_out[3 * S + k] = f.ux;
+      hist_out[4 * S + k] = f.uy;
       if (FINAL)
         final_node<R, MODE>(D, k, S, 0, hm.drho, f.rho, f.ux, f.uy, nullptr, ux_prev, uy_prev,
                             part, plo);
     } else {
       const R sl = Arith<R>::source(l, D, Axx, Axy, Ayy, Fxx, Fxy, Fyy, G);
       collide_cde<R, false>(D, k, S, dst, l, cm, f, sl, So, uxo, uyo, Fx, Fy, G);
-      hist[(size_t)l * S + k] = sl;
+      ((R*)D.hist_out)[(size_t)l * S + k] = sl;
       if (FINAL) {
         const R dphi[3] = {s_phi[0][lane], s_phi[1][lane], s_phi[2][lane]};
         final_node<R, MODE>(D, k, S, role, R(0), f.rho, f.ux, f.uy, dphi, 0.0, 0.0, part, plo);
