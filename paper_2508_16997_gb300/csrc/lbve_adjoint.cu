@@ -38,7 +38,10 @@ template <typename R, int MODE, bool OPEN, bool PUSH>
 static void run_pass(int pass, const InstDev* d, const AdjArgs<R>& A, int blocks, cudaStream_t st) {
   switch (pass) {
     case 0: adj_moments<R, MODE, OPEN><<<blocks, 256, 0, st>>>(d, A); break;
-    case 1: adj_local<R, MODE, OPEN, PUSH><<<blocks, 256, 0, st>>>(d, A); break;
+    case 1:
+      adj_local<R, MODE, OPEN, PUSH>
+          <<<blocks * (256 / kAdjLocalThreads), kAdjLocalThreads, 0, st>>>(d, A);
+      break;
     case 2: adj_gather<R, MODE, OPEN, PUSH><<<blocks, 256, 0, st>>>(d, A); break;
     case 4: adj_column<R, MODE><<<blocks, 256, 0, st>>>(d, A); break;
     default: adj_pull<R><<<blocks, 256, 0, st>>>(d, A); break;

@@ -534,10 +534,13 @@ __device__ __forceinline__ void push_lambda(const InstDev& D, R* __restrict__ la
 }
 
 // Pass 1: local reverse of the collision, source, history and CNEBB.
-// float32: a budget of 128 registers (two CTAs per SM) trades a few spills
-// for twice the warps in flight; float64 keeps its full register file.
+// float32: a budget of 128 registers trades a few spills for twice the warps in
+// flight (gradient of 200 steps at 512^2: 21.6 ms; at 80 or 96 registers 25.0 and
+// 22.7); float64 keeps its full register file, and two 128-thread CTAs fit an SM
+// where one of 256 did (50 steps at 128^2: 6.1 -> 5.0 ms).
+constexpr int kAdjLocalThreads = 128;
 template <typename R, int MODE, bool OPEN, bool PUSH>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1)
+__global__ void __launch_bounds__(kAdjLocalThreads, sizeof(R) == 4 ? 4 : 1)
     adj_local(const InstDev* __restrict__ Dp, AdjArgs<R> A) {
   const InstDev& D = *Dp;
   const int nx = D.nx, ny = D.ny, S = D.stride, n = nx * ny;

@@ -1818,7 +1818,8 @@ extern "C" int lbve_adjoint_step_ex(lbve_handle* h, int32_t inst, const double* 
   const int nmt = (int)mtiles.size();
   auto launch_tiles = [&](size_t at, int mode, int flags) -> bool {
     const int nt = h->plan.threads[q.list];
-    if (launch_step(prec, nt, d_desc + at, d_tiles, q.ntiles, 0, mode, flags, d_partials, st))
+    if (launch_step(prec, nt, d_desc + at, d_tiles, q.ntiles, 0, mode,
+                    flags | (masked || open ? 0 : kDependent), d_partials, st))
       return false;
     if (nmt > 0 &&
         launch_step(prec, nt, d_desc + at, d_mtiles, nmt, 0, mode, flags, d_partials, st, 1))
