@@ -137,7 +137,7 @@ struct InstPlan {
 struct Plan {
   std::vector<InstPlan> inst;
   size_t off_insts, off_tiles[kLists], off_partials, off_totals, off_flags, off_geo, total;
-  int ntiles[kLists], nslots;
+  int ntiles[kLists], nslots, max_slots;  // max_slots: of any instance
   int cap_tiles[kLists];  // tile-table capacity: the most tiles any tile width gives
   int threads[kLists];    // CTA size of each list's step launches
   size_t off_mtiles[kLists], off_walls[kLists], off_wrec[kLists], off_cols[kLists];
@@ -258,7 +258,7 @@ Plan make_plan(const lbve_params* p, int n) {
     pl.cap_tiles[q.list] += (int)max_tiles(p[i]);
   }
   // partial-record slots: [list 0 | list 1]
-  pl.nslots = 0;
+  pl.nslots = pl.max_slots = 0;
   for (int l = 0; l < kLists; ++l) pl.nslots += pl.ntiles[l];
   for (int i = 0; i < n; ++i) {
     InstPlan& q = pl.inst[i];
@@ -266,6 +266,7 @@ Plan make_plan(const lbve_params* p, int n) {
     for (int l = 0; l < q.list; ++l) base += pl.ntiles[l];
     q.slot_begin = base + q.tile_begin;
     q.nslots = q.ntiles;
+    pl.max_slots = std::max(pl.max_slots, q.nslots);
   }
   pl.off_insts = off;
   off = align_up(off + sizeof(InstDev) * n, kAlign);
@@ -944,8 +945,9 @@ static int stage_geometry(lbve_handle* h, int32_t inst, const uint8_t* solid_mas
 static int init_geometry(lbve_handle* h, int32_t n, const int32_t* ids, const int32_t* what) {
   if (n <= 0) return LBVE_OK;
   std::vector<int32_t> geo(2 * (size_t)n);
-  int max_nodes = 1;
+  int max_nodes = 1, max_slots = 0;
   for (int32_t j = 0; j < n; ++j) {
+    max_slots = std::max(max_slots, h->plan.inst[ids[j]].nslots);
     geo[j] = ids[j];
     geo[n + j] = what[j];
     max_nodes = std::max(max_nodes, h->p[ids[j]].nx * h->p[ids[j]].ny);
@@ -994,7 +996,8 @@ static int init_geometry(lbve_handle* h, int32_t n, const int32_t* ids, const in
                     kModeInit, kFinal, h->d_partials, h->stream, 1))
       return cuda_fail(cudaGetLastError(), "masked init kernel launch");
   }
-  if (launch_reduce(h->d_insts, 0, n, h->d_partials, h->d_totals, h->d_flags, h->stream, h->d_geo))
+  if (launch_reduce(h->d_insts, 0, n, max_slots, h->d_partials, h->d_totals, h->d_flags, h->stream,
+                    h->d_geo))
     return cuda_fail(cudaGetLastError(), "reduce launch");
   return LBVE_OK;
 }
@@ -1131,7 +1134,8 @@ int lbve_step(lbve_handle* h, int64_t n_steps) {
   int rc = launch_one_step(h, h->parity, kFinal, h->stream);
   if (rc) return rc;
   h->parity ^= 1;
-  if (launch_reduce(h->d_insts, 0, h->n, h->d_partials, h->d_totals, h->d_flags, h->stream))
+  if (launch_reduce(h->d_insts, 0, h->n, h->plan.max_slots, h->d_partials, h->d_totals, h->d_flags,
+                    h->stream))
     return cuda_fail(cudaGetLastError(), "reduce launch");
   for (int i = 0; i < h->n; ++i) h->t[i] += n_steps;
   return LBVE_OK;

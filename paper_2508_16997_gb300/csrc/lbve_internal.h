@@ -212,9 +212,10 @@ struct AdjArgsRaw {
 int launch_adjoint(int prec, int mode, int pass, const InstDev* d_desc, const AdjArgsRaw& a,
                    int n_nodes, void* stream);
 // Totals of n_insts instances: ids[0..n_insts-1] (device), or first_inst..
-// first_inst + n_insts - 1 when d_ids is null.
-int launch_reduce(const InstDev* d_insts, int first_inst, int n_insts, const double* d_partials,
-                  double* d_totals, int32_t* d_flags, void* stream,
+// first_inst + n_insts - 1 when d_ids is null.  max_slots: the most partial records
+// of any of them (their records are folded in place).
+int launch_reduce(const InstDev* d_insts, int first_inst, int n_insts, int max_slots,
+                  double* d_partials, double* d_totals, int32_t* d_flags, void* stream,
                   const int32_t* d_ids = nullptr);
 // Staged inputs of the list entries j < n_list (instance d_ids[j], d_what[j]
 // bit 0 force staged in pop[parity], bit 1 initial fields staged in

@@ -91,28 +91,72 @@ int launch_step(int prec, int threads, const InstDev* d_insts, const TileDev* d_
   return -1;
 }
 
-// One CTA per instance: sum (max for the residual) the partial records of the
-// instance's tiles, and the wall-pass records of its mask walls, in a fixed
-// order, so totals are bit-reproducible.  CTA b takes instance ids[b], or
-// first_inst + b without a list.  Warp j of the 16 reduces total j: each lane
-// runs over every 32nd record, then the warp folds its lanes by shuffles
-// (no block-wide barrier: GB300 issues float64 additions slowly, so the
-// sums are spread over warps instead of levels of a shared-memory tree).
+// Totals in two stages of a fixed order, so that they are bit-reproducible.
+// reduce_chunks_kernel: each CTA folds kReduceChunk consecutive records of an
+// instance into the first of them (only instances with more than two chunks;
+// blockIdx.y is the list entry).  Thread (g, j) sums value j of every 32nd
+// record: a warp reads whole lines.  reduce_kernel: one CTA per instance sums
+// (max for the residual) what is left and the wall-pass records of its mask
+// walls; warp j of the 16 reduces total j, each lane over every 32nd record, then
+// the warp folds its lanes by shuffles (no block-wide barrier: GB300 issues
+// float64 additions slowly, so the sums are spread over warps instead of levels
+// of a shared-memory tree).  With reduce_kernel alone one CTA walked the 43,700
+// records of a 2048^2 grid in 450 us, 8 % of a 20-step call.
+// List entry b is instance ids[b], or first_inst + b without a list.
 constexpr int kReduceThreads = 32 * kTotals;
+constexpr int kReduceChunk = 256;
 static_assert(kTotals == kDrag + 2, "one warp per total");
+static_assert(kPartial == 16 && kReduceThreads == 32 * kPartial, "thread (g, j) of a chunk");
+
+__device__ __forceinline__ bool in_chunks(const InstDev& D) {
+  return D.slot_end - D.slot_begin > 2 * kReduceChunk;
+}
+
+__global__ void __launch_bounds__(kReduceThreads)
+    reduce_chunks_kernel(const InstDev* __restrict__ insts, int first_inst,
+                         const int32_t* __restrict__ ids, double* __restrict__ partials) {
+  const InstDev& D = insts[ids ? ids[blockIdx.y] : first_inst + blockIdx.y];
+  const int begin = D.slot_begin + blockIdx.x * kReduceChunk;
+  if (!in_chunks(D) || begin >= D.slot_end) return;
+  const int n = min(kReduceChunk, D.slot_end - begin);
+  const int j = threadIdx.x & 15, g = threadIdx.x >> 4;
+  const bool is_max = j == kResid;
+  double* __restrict__ rec = partials + (size_t)begin * kPartial;
+  double v = 0.0;
+  if (j < kDrag)
+    for (int r = g; r < n; r += 32) {
+      const double p = rec[r * kPartial + j];
+      v = is_max ? fmax(v, p) : v + p;
+    }
+  __shared__ double s[32][kPartial];
+  s[g][j] = v;
+  __syncthreads();
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    if (g < o) {
+      const double w = s[g + o][j];
+      s[g][j] = v = is_max ? fmax(v, w) : v + w;
+    }
+    __syncthreads();
+  }
+  if (g == 0 && j < kDrag) rec[j] = v;
+}
+
 __global__ void __launch_bounds__(kReduceThreads) reduce_kernel(const InstDev* __restrict__ insts,
                                                                 int first_inst,
                                                                 const int32_t* __restrict__ ids,
+                                                                bool chunks,
                                                                 const double* __restrict__ partials,
                                                                 double* __restrict__ totals,
                                                                 int32_t* __restrict__ flags) {
   const int inst = ids ? ids[blockIdx.x] : first_inst + blockIdx.x;
   const InstDev& D = insts[inst];
   const int j = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int step = chunks && in_chunks(D) ? kReduceChunk : 1;
   const bool is_max = j == kResid;
   double v = 0.0;
   if (j < kDrag)
-    for (int q = D.slot_begin + lane; q < D.slot_end; q += 32) {
+    for (int q = D.slot_begin + lane * step; q < D.slot_end; q += 32 * step) {
       const double p = partials[(size_t)q * kPartial + j];
       v = is_max ? fmax(v, p) : v + p;
     }
@@ -131,12 +175,17 @@ __global__ void __launch_bounds__(kReduceThreads) reduce_kernel(const InstDev* _
   }
 }
 
-int launch_reduce(const InstDev* d_insts, int first_inst, int n_insts, const double* d_partials,
-                  double* d_totals, int32_t* d_flags, void* stream, const int32_t* d_ids) {
+int launch_reduce(const InstDev* d_insts, int first_inst, int n_insts, int max_slots,
+                  double* d_partials, double* d_totals, int32_t* d_flags, void* stream,
+                  const int32_t* d_ids) {
   if (n_insts <= 0) return 0;
-  reduce_kernel<<<n_insts, kReduceThreads, 0, (cudaStream_t)stream>>>(d_insts, first_inst, d_ids,
-                                                                      d_partials, d_totals,
-                                                                      d_flags);
+  cudaStream_t st = (cudaStream_t)stream;
+  const bool chunks = max_slots > 2 * kReduceChunk && n_insts <= 65535;  // grid y limit
+  if (chunks)
+    reduce_chunks_kernel<<<dim3((max_slots + kReduceChunk - 1) / kReduceChunk, n_insts),
+                           kReduceThreads, 0, st>>>(d_insts, first_inst, d_ids, d_partials);
+  reduce_kernel<<<n_insts, kReduceThreads, 0, st>>>(d_insts, first_inst, d_ids, chunks, d_partials,
+                                                    d_totals, d_flags);
   return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;  // the caller reads and clears it
 }
 
