@@ -151,7 +151,8 @@ struct Plan {
 // threads where that of a 32 x 2 tile (68, 132) takes two or three (128^2 mill
 // 15.3 -> 13.3 us per step, 192^2 21.2 -> 19.3).
 int default_tile_tx(const lbve_params& p, int threads = kThreads) {
-  const int w = threads <= kThreads64Small ? kTileTXTiny : kTileTX;
+  const int w = threads <= kThreads64Small ? kTileTXTiny
+                : threads == kThreads64Mid ? kTileTXMid : kTileTX;
   return p.nx >= w ? w : p.nx;
 }
 
@@ -178,6 +179,8 @@ int64_t max_tiles(const lbve_params& p) {
   int64_t m = 0;
   for (int TX = 1; TX <= std::min(tile_tx_max(p.precision), p.nx); ++TX) {
     m = std::max(m, tiles_for(p, TX, threads_of(p.precision)));
+    if (p.precision == LBVE_FP64 && TX <= kThreads64Mid / 2)
+      m = std::max(m, tiles_for(p, TX, kThreads64Mid));
     if (p.precision == LBVE_FP64 && TX <= kThreads64Small / 2)
       m = std::max(m, tiles_for(p, TX, kThreads64Small));
     if (p.precision == LBVE_FP64 && TX <= kThreads64Tiny / 2)
@@ -186,27 +189,31 @@ int64_t max_tiles(const lbve_params& p) {
   return m;
 }
 
-// CTA size of the float64 list.  The FP64 pipe bounds the float64 step, so a
-// batch whose 256-thread tiles would not give every SM one tile leaves SMs
-// idle while the others work through 256 nodes each; 64-thread tiles spread
-// the same nodes over four times as many CTAs, and one-warp tiles over eight
-// times as many when even the 64-thread tiles number fewer than the SMs.
-// Chosen from the parameters alone (the workspace plan needs no device): the
-// smallest size whose larger neighbour would leave SMs without a tile, as
-// long as no float64 instance asks for a tile wider than half the CTA.
+// CTA size of the float64 list.  The FP64 pipe bounds the float64 step, so SMs
+// without a tile, or a last wave that few of them work through, cost as much as
+// full ones.  By the number of 256-thread tiles of the batch:
+//   >= 5 per SM  256 threads (512^2 mill 109 us per step, 114 with 128);
+//   >= 1 per SM  128 threads (200^2 25.7 us, 32.1 with 256; 300^2 42.1, 48.5;
+//                400^2 71.1, 77.7);
+//   below        64 threads, and one-warp tiles (one lattice per warp) when
+//                even the 64-thread tiles number fewer than the SMs.
+// Chosen from the parameters alone (the workspace plan needs no device), as long
+// as no float64 instance asks for a tile wider than half the CTA.
 int fp64_threads(const lbve_params* p, int n) {
   int64_t t256 = 0, t64 = 0;
   int maxtx = 0;
   bool any = false;
   for (int i = 0; i < n; ++i) {
     if (p[i].precision != LBVE_FP64) continue;
-    if (p[i].tile_tx > kThreads64Small / 2) return kThreads64;
+    if (p[i].tile_tx > kThreads64Mid / 2) return kThreads64;
     any = true;
     maxtx = std::max(maxtx, (int)p[i].tile_tx);
     t256 += tiles_for(p[i], tile_width(p[i], kThreads64), kThreads64);
-    t64 += tiles_for(p[i], tile_width(p[i], kThreads64Small), kThreads64Small);
+    if (p[i].tile_tx <= kThreads64Small / 2)
+      t64 += tiles_for(p[i], tile_width(p[i], kThreads64Small), kThreads64Small);
   }
-  if (!any || t256 >= kNumSMs) return kThreads64;
+  if (!any || t256 >= 5 * kNumSMs) return kThreads64;
+  if (maxtx > kThreads64Small / 2 || t256 >= kNumSMs) return kThreads64Mid;
   if (maxtx > kThreads64Tiny / 2 || t64 >= kNumSMs) return kThreads64Small;
   return kThreads64Tiny;
 }

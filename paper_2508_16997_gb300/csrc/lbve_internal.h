@@ -22,6 +22,11 @@ int set_error(int code, const char* fmt, ...) __attribute__((format(printf, 2, 3
 #ifndef LBVE_THREADS_FP64
 #define LBVE_THREADS_FP64 256
 #endif
+// Float64 batches of a few 256-thread tiles per SM run 128-thread CTAs (16 x 8
+// tiles): the last wave of 256-thread tiles costs them more than the larger halo.
+#ifndef LBVE_THREADS_FP64_MID
+#define LBVE_THREADS_FP64_MID 128
+#endif
 #ifndef LBVE_THREADS_FP64_SMALL
 #define LBVE_THREADS_FP64_SMALL 64
 #endif
@@ -36,9 +41,11 @@ int set_error(int code, const char* fmt, ...) __attribute__((format(printf, 2, 3
 #endif
 constexpr int kThreads = LBVE_THREADS;          // float32 step kernel
 constexpr int kThreads64 = LBVE_THREADS_FP64;   // float64 step kernel
+constexpr int kThreads64Mid = LBVE_THREADS_FP64_MID;      // float64, mid-size batches
 constexpr int kThreads64Small = LBVE_THREADS_FP64_SMALL;  // float64, small batches
 constexpr int kThreads64Tiny = LBVE_THREADS_FP64_TINY;    // float64, tiny batches
 constexpr int kTileTXTiny = 8;  // default tile width of the one- and two-warp float64 CTAs
+constexpr int kTileTXMid = 16;  // default tile width of the 128-thread float64 CTAs
 constexpr int kNumSMs = 152;  // GB300; sizes the small-batch choice only
 constexpr int kTileTX = LBVE_TILE_TX;   // default tile width (nodes along x) for nx >= kTileTX
 // threads per CTA (for float64, the size of all but small batches) and the
@@ -163,7 +170,7 @@ struct alignas(16) ColTask {
 // Launchers implemented in lbve_kernels.cu (templated over float/double).
 enum : int { kModeStep = 0, kModeInit = 1 };
 
-// threads: CTA size of the tiles (kThreads for float32; kThreads64,
+// threads: CTA size of the tiles (kThreads for float32; kThreads64, kThreads64Mid,
 // kThreads64Small or kThreads64Tiny for float64).  masked = 0 runs the plain kernel (which
 // skips masked tiles), 1 the masked variant.
 int launch_step(int prec, int threads, const InstDev* d_insts, const TileDev* d_tiles,

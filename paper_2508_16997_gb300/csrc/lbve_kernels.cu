@@ -64,6 +64,9 @@ int launch_step(int prec, int threads, const InstDev* d_insts, const TileDev* d_
   if (prec == 0 && threads == kThreads64)
     return launch_step_m<double, kThreads64, kThreads64>(d_insts, d_tiles, n_tiles, parity, mode, flags,
                                              d_partials, st, masked);
+  if (prec == 0 && threads == kThreads64Mid)
+    return launch_step_m<double, kThreads64Mid, kThreads64Mid>(
+        d_insts, d_tiles, n_tiles, parity, mode, flags, d_partials, st, masked);
   if (prec == 0 && threads == kThreads64Tiny) {
     // tiles of at most 32 nodes: the time steps of plain tiles spread each
     // node over four warps (one lattice each), the rest runs one warp a tile

@@ -1032,7 +1032,7 @@ struct MinBlocks {
       std::is_same<R, df32>::value
           ? LBVE_DF32_MIN_BLOCKS
           : sizeof(R) == 4 ? (MASKED ? LBVE_FP32_MASKED_MIN_BLOCKS : LBVE_FP32_MIN_BLOCKS)
-                           : (NT <= 32 ? 2 : NT <= 64 ? 4 : MASKED && NT < 256 ? 1 : 512 / NT);
+                           : (NT <= 32 ? 2 : NT <= 64 ? 4 : MASKED && NT < 256 ? 512 / NT / 4 : 512 / NT);
 };
 
 // Open channels: nodes of the inlet (x = 0) and outlet (x = nx - 1) columns

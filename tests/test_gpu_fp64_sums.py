@@ -65,3 +65,17 @@ def test_overflow_is_reported(lbve):
     s = lbve.Simulation([inst], precision=lbve.LBVE_FP64, init_fields=[init])
     s.step(2)
     assert s.status()[0] & 1
+
+
+@pytest.mark.parametrize("nx,ny,periodic", [(200, 200, True), (203, 197, False), (130, 400, True)])
+def test_mid_size_cta_bit_identical(lbve, nx, ny, periodic):
+    """152 to 759 tiles of 256 threads: the default 128-thread CTAs against the
+    256-thread ones that a 128-wide tile asks for, bit for bit."""
+    inst = wl.Instance(nx, ny, periodic, 0.5, 2.0, 1.0, 1e4, 0.05, 100.0, Fx=1e-5, Fy=-3e-6)
+    init = wl.random_fields(nx, ny, seed=4, du=1e-3)
+    runs = []
+    for tx in (0, 128):
+        s = lbve.Simulation([inst], precision=lbve.LBVE_FP64, init_fields=[init], tile_tx=tx)
+        s.step(20)
+        runs.append(s.fields(0))
+    np.testing.assert_array_equal(runs[0], runs[1])
