@@ -31,20 +31,37 @@ static AdjArgs<R> cast_args(const AdjArgsRaw& a) {
   return A;
 }
 
+template <typename R, typename K>
+static void launch(K kernel, int blocks, int threads, const InstDev* d, const AdjArgs<R>& A,
+                   cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(threads);
+  cfg.stream = st;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  // float64 passes of more than half an SM each would put early CTAs beside running
+  // ones on the same float64 pipe (128^2, 50 steps: 5.0 ms without, 6.0 with)
+  cfg.numAttrs = sizeof(R) == 4 || 2 * blocks <= kNumSMs ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, d, A);
+}
+
 // OPEN: the node passes' variant with an open channel's inlet and outlet
 // columns (one-sided x-differences there in every mode, the column pass's
 // completion in the step modes).
 template <typename R, int MODE, bool OPEN, bool PUSH>
 static void run_pass(int pass, const InstDev* d, const AdjArgs<R>& A, int blocks, cudaStream_t st) {
   switch (pass) {
-    case 0: adj_moments<R, MODE, OPEN><<<blocks, 256, 0, st>>>(d, A); break;
+    case 0: launch(adj_moments<R, MODE, OPEN>, blocks, 256, d, A, st); break;
     case 1:
-      adj_local<R, MODE, OPEN, PUSH>
-          <<<blocks * (256 / kAdjLocalThreads), kAdjLocalThreads, 0, st>>>(d, A);
+      launch(adj_local<R, MODE, OPEN, PUSH>, blocks * (256 / kAdjLocalThreads), kAdjLocalThreads, d,
+             A, st);
       break;
-    case 2: adj_gather<R, MODE, OPEN, PUSH><<<blocks, 256, 0, st>>>(d, A); break;
-    case 4: adj_column<R, MODE><<<blocks, 256, 0, st>>>(d, A); break;
-    default: adj_pull<R><<<blocks, 256, 0, st>>>(d, A); break;
+    case 2: launch(adj_gather<R, MODE, OPEN, PUSH>, blocks, 256, d, A, st); break;
+    case 4: launch(adj_column<R, MODE>, blocks, 256, d, A, st); break;
+    default: launch(adj_pull<R>, blocks, 256, d, A, st); break;
   }
 }
 

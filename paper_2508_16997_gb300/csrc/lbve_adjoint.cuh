@@ -20,6 +20,9 @@
 //               writes lambda of the hydro pulls, accumulates dL/dF
 //   adj_pull    reverse pull into lambda_t's populations (masks and open columns
 //               only: else the first two passes write lambda_t themselves)
+// The passes launch with the programmatic dependency of the step kernels: each
+// starts while the one before it ends and waits for it before the first access
+// (512^2, 200 steps, float32: 21.6 -> 19.5 ms; 48^2, 60 steps: 1.7 ms).
 // A fourth kernel (adj_moments) recomputes rho, u of the forward state so the
 // gather can read its neighbours.  Open channels add a fifth between the
 // gather and the pull (adj_column): the inlet and outlet nodes' completed
@@ -330,6 +333,8 @@ __device__ __forceinline__ void adj_hydro_node(const InstDev& D, const AdjArgs<R
 // rho, u of every node of the forward state (for the neighbours' gradients).
 template <typename R, int MODE, bool OPEN>
 __global__ void adj_moments(const InstDev* __restrict__ Dp, AdjArgs<R> A) {
+  start_next_kernel();
+  wait_previous_kernel();
   const InstDev& D = *Dp;
   const int n = D.nx * D.ny;
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -542,6 +547,8 @@ constexpr int kAdjLocalThreads = 128;
 template <typename R, int MODE, bool OPEN, bool PUSH>
 __global__ void __launch_bounds__(kAdjLocalThreads, sizeof(R) == 4 ? 4 : 1)
     adj_local(const InstDev* __restrict__ Dp, AdjArgs<R> A) {
+  start_next_kernel();
+  wait_previous_kernel();
   const InstDev& D = *Dp;
   const int nx = D.nx, ny = D.ny, S = D.stride, n = nx * ny;
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -902,6 +909,8 @@ __global__ void __launch_bounds__(kAdjLocalThreads, sizeof(R) == 4 ? 4 : 1)
 // accumulates dL/dF.
 template <typename R, int MODE, bool OPEN, bool PUSH>
 __global__ void adj_gather(const InstDev* __restrict__ Dp, AdjArgs<R> A) {
+  start_next_kernel();
+  wait_previous_kernel();
   const InstDev& D = *Dp;
   const int nx = D.nx, ny = D.ny, S = D.stride, n = nx * ny;
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1008,6 +1017,8 @@ __global__ void adj_gather(const InstDev* __restrict__ Dp, AdjArgs<R> A) {
 // entries are then cleared: it pulls nothing.
 template <typename R, int MODE>
 __global__ void adj_column(const InstDev* __restrict__ Dp, AdjArgs<R> A) {
+  start_next_kernel();
+  wait_previous_kernel();
   const InstDev& D = *Dp;
   const int nx = D.nx, ny = D.ny, S = D.stride, n = nx * ny;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1124,6 +1135,8 @@ __global__ void adj_column(const InstDev* __restrict__ Dp, AdjArgs<R> A) {
 // outlet reads the (cleared) entries of the far open column: zero.
 template <typename R>
 __global__ void adj_pull(const InstDev* __restrict__ Dp, AdjArgs<R> A) {
+  start_next_kernel();
+  wait_previous_kernel();
   const InstDev& D = *Dp;
   const int nx = D.nx, S = D.stride, n = nx * D.ny;
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
