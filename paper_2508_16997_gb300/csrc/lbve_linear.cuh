@@ -25,8 +25,9 @@
 // 2.3e-12, 1.6e-12.  Ties to even take 5 instructions more per input and no
 // smaller error (5.0e-14, 3.2e-13, 1.5e-12; the mix 5 % slower).
 // Results round to nearest even.  Exact zeros stay zero.  Inputs of exponent
-// 2^1009 and above (infinities and NaN among them) give NaN; below 2^-895 the
-// last place is 2^-953 whatever the largest value (kFixMinE).
+// 2^1020 and above (infinities and NaN among them) give NaN, where float64
+// additions would still have a finite sum up to 2^1024; below 2^-959 the last place
+// is 2^-1017 whatever the largest value (kFixMinE).
 //   The functions also compile for the host, where the tests compare them with
 // exact arithmetic.
 #pragma once
@@ -99,8 +100,12 @@ LBVE_HD int leading_zeros(uint64_t v) {
 }
 
 // ---- block fixed point -------------------------------------------------------
-constexpr int kFixMinE = 128 << 20;   // smallest block exponent (in place, biased)
-constexpr int kFixMaxE = 2032 << 20;  // from here on: not finite
+// Smallest block exponent (in place, biased): the smallest result, a quarter of
+// the unit 2^-1017, is still a normal number.
+constexpr int kFixMinE = 64 << 20;
+// Not finite from here on: the largest sum, that of n_xx over 15 inputs, would
+// leave the range of float64.
+constexpr int kFixMaxE = 2043 << 20;
 
 // Exponent field of a float64 value, in place.
 LBVE_HD int fix_exponent(double d) { return high_word(d) & 0x7ff00000; }
@@ -124,7 +129,7 @@ LBVE_HD int64_t fix_from(double d, int block) {
   const int hi = high_word(d);
   const unsigned lo = low_word(d);
   const unsigned vh = top_word(hi, lo) | 0x80000000u;  // leading bit at 63
-  const unsigned sh = (unsigned)(block + (4 << 20) - (hi & 0x7ff00000)) >> 20;
+  const unsigned sh = ((unsigned)block + (4u << 20) - ((unsigned)hi & 0x7ff00000u)) >> 20;
   const uint64_t r = shift_right(((uint64_t)vh << 32) | (lo << 11), sh);
   const int64_t s = (int64_t)(hi >> 31);
   return (int64_t)((r ^ (uint64_t)s) + 1) >> 1;
@@ -141,8 +146,8 @@ LBVE_HD double fix_to(int64_t v, int block, int nan) {
   const uint64_t q = w >> 11;
   const unsigned up = (((unsigned)w & 0x7ffu) + ((unsigned)q & 1u) + 0x3ffu) >> 11;
   // bit 52 of q adds the implicit one to the exponent field
-  const int t = a == 0 ? 0 : block + ((4 + SCALE) << 20) - (k << 20);
-  const uint64_t r = q + ((uint64_t)(uint32_t)t << 32) + up;
+  const unsigned t = a == 0 ? 0u : (unsigned)block + ((4u + SCALE) << 20) - ((unsigned)k << 20);
+  const uint64_t r = q + ((uint64_t)t << 32) + up;
   return from_words((int)(r >> 32) | (s & (int)0x80000000) | nan, (unsigned)r);
 }
 
