@@ -417,9 +417,11 @@ __device__ __forceinline__ double mad(double a, double b, double c) { return fma
 
 // 1 / v by one step of the cubically convergent iteration x (1 + e + e^2),
 // e = 1 - v x (Householder's method), from the float32 approximate
-// reciprocal: three float64 instructions where the division takes about nine,
-// error below 2^-52 of the result.  Outside [2^-100, 2^100] (and for NaN) it
-// divides.
+// reciprocal: three float64 instructions where the division takes about nine.
+// x is off by at most 2^-22 of its size (v truncated to 24 bits, the approximation
+// within 2^-23), so the step leaves 2^-66 and the result is within 1/2 + 2^-12
+// units of its last place (the division: 1/2; one of some 10^4 results
+// differs from it, by one unit).  Outside [2^-100, 2^101) and for NaN it divides.
 __device__ __forceinline__ double recip(double v) {
   const int hi = __double2hiint(v), lo = __double2loint(v);
   const unsigned e = ((unsigned)hi >> 20) & 0x7ffu;

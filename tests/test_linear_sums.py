@@ -189,3 +189,38 @@ def test_device_equals_host(gpu_probe, kind, third):
     dev = sums(gpu_probe.probe_sums_device, kind, third, a)
     np.testing.assert_array_equal(dev, host)  # NaN equals NaN
     np.testing.assert_array_equal(np.signbit(dev[dev == 0]), np.signbit(host[host == 0]))
+
+
+@pytest.mark.gpu
+def test_reciprocal(gpu_probe):
+    """1 / v: within 1/2 + 2^-12 units of the last place over [2^-100, 2^101), the
+    division itself outside.  x has at most 2^-22 relative error (v truncated to
+    24 bits, rcp.approx within 2^-23), so the cubic step leaves 2^-66, its two
+    inner roundings 2^-75 each: together below 2^-13 units before the last
+    rounding."""
+    rng = np.random.default_rng(5)
+    n = 200000
+    near = np.concatenate([1.0 + rng.uniform(-0.1, 0.1, n // 2), rng.uniform(1.0, 2.0, n // 2)])
+    wide = np.ldexp(rng.uniform(1.0, 2.0, n), rng.integers(-100, 101, n))
+    edges = np.array([np.nextafter(np.ldexp(1.0, k), s) for k in range(-100, 101)
+                      for s in (0.0, np.inf)] + [np.ldexp(1.0, k) for k in range(-100, 101)])
+    edges = edges[(edges >= 2.0 ** -100) & (edges < 2.0 ** 101)]
+    v = np.concatenate([near, wide, edges])
+    v[::3] *= -1.0
+    out = np.empty_like(v)
+    assert gpu_probe.probe_recip_device(_ptr(v), _ptr(out), ctypes.c_longlong(v.size)) == 0
+    # exact in integers: |out v - 1| against ulp(out) v / 2 (1 + 2^-11), every 7th value
+    for a, r in zip(v[::7], out[::7]):
+        exact = 1 / Fraction(a)
+        assert abs(Fraction(r) - exact) <= Fraction(float(np.spacing(abs(r)))) * (
+            Fraction(1, 2) + Fraction(1, 2 ** 12)), a
+    # all of them against the correctly rounded quotient: at most one place off
+    assert (np.abs(out - 1.0 / v) <= np.spacing(np.abs(out))).all()
+
+    v = np.array([0.0, -0.0, np.inf, -np.inf, np.nan, 5e-324, -1e-310, np.finfo(float).tiny,
+                  np.finfo(float).max, np.ldexp(1.0, 101), -np.ldexp(1.5, 300),
+                  np.nextafter(2.0 ** -100, 0.0), -np.ldexp(1.1, -500)])
+    out = np.empty_like(v)
+    assert gpu_probe.probe_recip_device(_ptr(v), _ptr(out), ctypes.c_longlong(v.size)) == 0
+    with np.errstate(divide="ignore", over="ignore"):
+        np.testing.assert_array_equal(out, 1.0 / v)
