@@ -46,7 +46,7 @@ constexpr int kThreads64Small = LBVE_THREADS_FP64_SMALL;  // float64, small batc
 constexpr int kThreads64Tiny = LBVE_THREADS_FP64_TINY;    // float64, tiny batches
 constexpr int kTileTXTiny = 8;  // default tile width of the one- and two-warp float64 CTAs
 constexpr int kTileTXMid = 16;  // default tile width of the 128-thread float64 CTAs
-constexpr int kNumSMs = 152;  // GB300; sizes the small-batch choice only
+constexpr int kNumSMs = 152;  // GB300; sizes the CTA and launch choices only
 constexpr int kTileTX = LBVE_TILE_TX;   // default tile width (nodes along x) for nx >= kTileTX
 // threads per CTA (for float64, the size of all but small batches) and the
 // widest tile a caller may ask for, by precision (0 = float64, 1 = float32

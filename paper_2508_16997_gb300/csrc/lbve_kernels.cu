@@ -7,7 +7,7 @@
 
 namespace lbve {
 
-template <typename R, int MODE, bool FINAL, bool MASKED, int NT>
+template <typename R, int MODE, bool FINAL, bool MASKED, int NT, int MB>
 static void launch_step_k(const InstDev* d_insts, const TileDev* d_tiles, int n_tiles, int parity,
                           double* d_partials, cudaStream_t st, bool dependent = false) {
   cudaLaunchConfig_t cfg = {};
@@ -20,40 +20,63 @@ static void launch_step_k(const InstDev* d_insts, const TileDev* d_tiles, int n_
   attr.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &attr;
   cfg.numAttrs = dependent && overlaps_steps<R, MODE, MASKED>() ? 1 : 0;
-  cudaLaunchKernelEx(&cfg, step_kernel<R, MODE, FINAL, MASKED, NT>, d_insts, d_tiles, parity,
+  cudaLaunchKernelEx(&cfg, step_kernel<R, MODE, FINAL, MASKED, NT, MB>, d_insts, d_tiles, parity,
                      d_partials);
 }
 
-template <typename R, bool MASKED, int NT>
+template <typename R, bool MASKED, int NT, int MB = MinBlocks<R, MASKED, NT>::value>
 static int launch_step_t(const InstDev* d_insts, const TileDev* d_tiles, int n_tiles, int parity,
                          int mode, int flags, double* d_partials, cudaStream_t st) {
   if (n_tiles <= 0) return 0;
   const bool fin = (flags & kFinal) != 0, dep = (flags & kDependent) != 0;
   if (mode == kModeStep) {
     if (fin)
-      launch_step_k<R, kModeStep, true, MASKED, NT>(d_insts, d_tiles, n_tiles, parity, d_partials,
-                                                    st, dep);
+      launch_step_k<R, kModeStep, true, MASKED, NT, MB>(d_insts, d_tiles, n_tiles, parity,
+                                                        d_partials, st, dep);
     else
-      launch_step_k<R, kModeStep, false, MASKED, NT>(d_insts, d_tiles, n_tiles, parity,
-                                                     d_partials, st, dep);
+      launch_step_k<R, kModeStep, false, MASKED, NT, MB>(d_insts, d_tiles, n_tiles, parity,
+                                                         d_partials, st, dep);
   } else {
-    launch_step_k<R, kModeInit, true, MASKED, NT>(d_insts, d_tiles, n_tiles, parity, d_partials,
-                                                  st);
+    launch_step_k<R, kModeInit, true, MASKED, NT, MB>(d_insts, d_tiles, n_tiles, parity,
+                                                      d_partials, st);
   }
   return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;  // the caller reads and clears it
 }
 
-// Masked tiles take more threads than nodes, so that other warps than those of
-// the nodes cover the halo ring, in one round (134 ring nodes of a 32 x 3
-// float32 tile, 48 of an 8 x 8 float64 one; wider rings loop): there are few such
-// tiles, and each is a serial chain (float32 10.8 -> 8.6 us, isolated).
-template <typename R, int NT, int NTM>
+// Masked tiles run in one of two shapes of the same kernel, with the same results.
+//   Few of them (a cylinder, the ends of an open channel): each is a serial chain
+//   that the step waits for, so it takes NTF threads, in float32 more than it has
+//   nodes (other warps than those of the nodes then cover the halo ring, in one
+//   round), with registers for MBF CTAs per SM, without spills.
+//   Many of them (every tile of a FENE or eq_p_G instance, domains full of solid
+//   nodes): nodes in flight per SM count, and they take the plain tiles' NT
+//   threads and as many CTAs as its register budget holds.
+// The line is one wave of the first shape: WAVE CTAs per SM (0: one shape only).
+// Microseconds per step, first / second shape:
+//   float32 (456 tiles): cylinders in open channels R = 16 (72 tiles) 9.5 / 10.9,
+//     R = 32 (154) 11.3 / 12.5, R = 64 (367) 38.1 / 38.9, R = 96 (650) 75.9 / 74.9;
+//     FENE-P mills 190^2 (384) 5.9 / 5.8, 200^2 (469) 8.4 / 6.1, 512^2 26.4 / 19.8,
+//     1024^2 125 / 92;
+//   float64, 128-thread CTAs (304 tiles): R = 20 (44 tiles) 34.7 / 41.3, R = 24 (58)
+//     50.4 / 49.5, R = 32 (78) 64.5 / 67.5, R = 39 (118) 100.7 / 101.1; FENE-P mills
+//     200^2 (325) 35.7 / 28.5, 384^2 85 / 70.
+// 64-thread float64 tiles keep their 64 threads: the ring (48 nodes at most) is one
+// round of them anyway (R = 16: 33 us per step, 40 with 128 threads; FENE-P 150^2:
+// 20 and 29).  One-warp tiles always take 64: the batches that run them have fewer
+// masked tiles than one wave (R = 8: 30.6 us, 31.7 with 32 threads).
+template <typename R, int NT, int NTF, int MBF, int WAVE>
 static int launch_step_m(const InstDev* d_insts, const TileDev* d_tiles, int n_tiles, int parity,
                          int mode, int flags, double* d_partials, cudaStream_t st, int masked) {
-  return masked ? launch_step_t<R, true, NTM>(d_insts, d_tiles, n_tiles, parity, mode, flags,
-                                             d_partials, st)
-                : launch_step_t<R, false, NT>(d_insts, d_tiles, n_tiles, parity, mode, flags,
-                                              d_partials, st);
+  if (!masked)
+    return launch_step_t<R, false, NT>(d_insts, d_tiles, n_tiles, parity, mode, flags, d_partials,
+                                       st);
+  if constexpr (WAVE > 0) {
+    if (n_tiles > WAVE * kNumSMs)
+      return launch_step_t<R, true, NT>(d_insts, d_tiles, n_tiles, parity, mode, flags, d_partials,
+                                        st);
+  }
+  return launch_step_t<R, true, NTF, MBF>(d_insts, d_tiles, n_tiles, parity, mode, flags,
+                                          d_partials, st);
 }
 
 // Only the CTA sizes the host plans are instantiated; any other is refused.
@@ -62,10 +85,10 @@ int launch_step(int prec, int threads, const InstDev* d_insts, const TileDev* d_
                 int masked) {
   cudaStream_t st = (cudaStream_t)stream;
   if (prec == 0 && threads == kThreads64)
-    return launch_step_m<double, kThreads64, kThreads64>(d_insts, d_tiles, n_tiles, parity, mode, flags,
-                                             d_partials, st, masked);
+    return launch_step_m<double, kThreads64, kThreads64, 2, 0>(d_insts, d_tiles, n_tiles, parity, mode,
+                                                            flags, d_partials, st, masked);
   if (prec == 0 && threads == kThreads64Mid)
-    return launch_step_m<double, kThreads64Mid, kThreads64Mid>(
+    return launch_step_m<double, kThreads64Mid, kThreads64Mid, 1, 2>(
         d_insts, d_tiles, n_tiles, parity, mode, flags, d_partials, st, masked);
   if (prec == 0 && threads == kThreads64Tiny) {
     // tiles of at most 32 nodes: the time steps of plain tiles spread each
@@ -79,15 +102,15 @@ int launch_step(int prec, int threads, const InstDev* d_insts, const TileDev* d_
                                                                     d_partials);
       return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;  // the caller reads and clears it
     }
-    return launch_step_m<double, kThreads64Tiny, 64>(d_insts, d_tiles, n_tiles, parity, mode, flags,
-                                                 d_partials, st, masked);
+    return launch_step_m<double, kThreads64Tiny, 64, 4, 0>(d_insts, d_tiles, n_tiles, parity, mode,
+                                                        flags, d_partials, st, masked);
   }
   if (prec == 0 && threads == kThreads64Small)
-    return launch_step_m<double, kThreads64Small, 128>(d_insts, d_tiles, n_tiles, parity, mode, flags,
-                                                  d_partials, st, masked);
+    return launch_step_m<double, kThreads64Small, kThreads64Small, 4, 0>(
+        d_insts, d_tiles, n_tiles, parity, mode, flags, d_partials, st, masked);
   if (prec == 1 && threads == kThreads)
-    return launch_step_m<float, kThreads, 160>(d_insts, d_tiles, n_tiles, parity, mode, flags,
-                                          d_partials, st, masked);
+    return launch_step_m<float, kThreads, 160, 3, 3>(d_insts, d_tiles, n_tiles, parity, mode, flags,
+                                                  d_partials, st, masked);
   if (prec == 2 && threads == kThreads && !masked)  // float32 pairs: plain tiles only
     return launch_step_t<df32, false, kThreads>(d_insts, d_tiles, n_tiles, parity, mode, flags,
                                                 d_partials, st);

@@ -1017,10 +1017,10 @@ __device__ __forceinline__ void collide_node(const InstDev& D, int k, int S, R* 
 // Resident CTAs per SM the register budget is sized for: the float32 step
 // is HBM-bound and wants more loads in flight; the float64 step is bound by
 // the FP64 pipe.
-// Masked tiles carry the mask's one-sided differences: a budget of 3 CTAs of
-// 160 threads per SM lets them keep their registers without spills.
+// Masked tiles carry the mask's one-sided differences: 5 CTAs of 96 threads per
+// SM (few of them run in another shape, launch_step_m).
 #ifndef LBVE_FP32_MASKED_MIN_BLOCKS
-#define LBVE_FP32_MASKED_MIN_BLOCKS 3
+#define LBVE_FP32_MASKED_MIN_BLOCKS 5
 #endif
 // Float64 CTAs: 256 threads two per SM (128 registers per thread).  The
 // 64- and one-warp CTAs serve batches with fewer tiles than 4 and 2 per SM,
@@ -1036,7 +1036,7 @@ struct MinBlocks {
       std::is_same<R, df32>::value
           ? LBVE_DF32_MIN_BLOCKS
           : sizeof(R) == 4 ? (MASKED ? LBVE_FP32_MASKED_MIN_BLOCKS : LBVE_FP32_MIN_BLOCKS)
-                           : (NT <= 32 ? 2 : NT <= 64 ? 4 : MASKED && NT < 256 ? 512 / NT / 4 : 512 / NT);
+                           : (NT <= 32 ? 2 : NT <= 64 ? 4 : 512 / NT);
 };
 
 // Open channels: nodes of the inlet (x = 0) and outlet (x = nx - 1) columns
@@ -1524,8 +1524,8 @@ __device__ __forceinline__ void process_tile(const InstDev* __restrict__ insts, 
 // TX * TY <= NT for every tile of the launch).  The plain variant leaves
 // masked tiles to the masked one (which runs over a separate list of just
 // those tiles).
-template <typename R, int MODE, bool FINAL, bool MASKED, int NT>
-__global__ void __launch_bounds__(NT, MinBlocks<R, MASKED, NT>::value)
+template <typename R, int MODE, bool FINAL, bool MASKED, int NT, int MB>
+__global__ void __launch_bounds__(NT, MB)
     step_kernel(const InstDev* __restrict__ insts, const TileDev* __restrict__ tiles,
                 int parity, double* __restrict__ partials) {
   static_assert(NT % 32 == 0 && NT >= 32, "whole warps; the final-step reduction reads 14 lanes");
