@@ -806,13 +806,12 @@ int lbve_create(const lbve_params* p, int32_t n, void* d_workspace, size_t bytes
     D.cd[kCoefMupLam] = c.mup / c.lambda;
     D.cd[kCoefInvL2] = p[i].model != 0 ? 1.0 / p[i].L2 : 0.0;
     D.cd[kCoefAfene] = p[i].model == 1 ? 1.0 / (1.0 - 2.0 / p[i].L2) : 1.0;
-    const double d = p[i].precision == LBVE_FP32_DEV ? 1.0 : 1.0 / 3.0;
-    D.cd[kCoefN1] = D.cd[kCoefCs1] * d / 3.0;
+    D.cd[kCoefN1] = D.cd[kCoefCs1] / 9.0;
     D.cd[kCoefN2] = D.cd[kCoefCs2] / 3.0;
     D.cd[kCoefHs2] = D.cd[kCoefHs1] / 2.0;
     D.cd[kCoefWx] = D.cd[kCoefMupLam] * D.cd[kCoefWs1];
-    D.cd[kCoefWd] = D.cd[kCoefWx] * d;
-    D.cd[kCoefP2] = D.cd[kCoefCp2] * d / 3.0;
+    D.cd[kCoefWd] = D.cd[kCoefWx] / 3.0;
+    D.cd[kCoefP2] = D.cd[kCoefCp2] / 9.0;
     D.model = p[i].model;
     D.gtilde = p[i].gtilde;
     D.t32 = q.TX == kTileTX && (!p[i].periodic_y || p[i].ny >= q.TY + 2);

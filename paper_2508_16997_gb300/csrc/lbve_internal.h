@@ -75,7 +75,7 @@ enum : int {
   kDependent = 2  // the launch may overlap the end of the step kernel before it
 };
 
-// Coefficient slots of InstDev::cd / InstDev::cf.
+// Coefficient slots of InstDev::cd, cf and cl.
 enum : int {
   kCoefFx = 0, kCoefFy,
   kCoefCs1,     // 1 - 1/tau_s1
@@ -89,15 +89,15 @@ enum : int {
   kCoefMupLam,  // mu_p/lambda
   kCoefInvL2,   // 1/L^2 of the FENE models (0 for Oldroyd-B)
   kCoefAfene,   // a = 1/(1 - 2/L^2) of FENE-P
-  // products the step uses; d = 1/3 for the 8-byte precisions, whose diagonal
-  // second-order terms carry the factor 1/3, 1 for float32
-  kCoefN1,      // (1 - 1/tau_s1) d / 3
-  kCoefN2,      // (1 - 1/tau_s2) / 3
-  kCoefHs2,     // (1 - 1/(2 tau_s1)) / 2
-  kCoefWd,      // mu_p / (lambda tau_s1) d
-  kCoefWx,      // mu_p / (lambda tau_s1)
-  kCoefP2,      // (1 - 1/tau_p2) d / 3
-  kNumCoef
+  kNumCoef,     // slots of cf and cl; the rest are products that only the
+                // float64 step reads, from cd
+  kCoefN1 = kNumCoef,  // (1 - 1/tau_s1) / 9
+  kCoefN2,             // (1 - 1/tau_s2) / 3
+  kCoefHs2,            // (1 - 1/(2 tau_s1)) / 2
+  kCoefWd,             // mu_p / (3 lambda tau_s1)
+  kCoefWx,             // mu_p / (lambda tau_s1)
+  kCoefP2,             // (1 - 1/tau_p2) / 9
+  kNumCoef64
 };
 
 // Everything a CTA needs about its instance.  Pointers are device addresses
@@ -122,7 +122,7 @@ struct alignas(16) InstDev {
   // Collision coefficients rounded once to float32 (cf), their float64
   // values (cd) and the low parts of the LBVE_DF32 pairs (cl = cd - cf), so
   // that no kernel converts precision per node.
-  float cf[20];
+  float cf[16];
   double* fields;                // [6][stride]  rho, ux, uy, Axx, Axy, Ayy (float64)
   const uint8_t* mask;           // [stride] 1 = solid node, or null (no mask)
   double* wall_rec;              // [wall_cap][kWallRec] final-step wall sums
@@ -134,10 +134,10 @@ struct alignas(16) InstDev {
                        // state's where states are kept (adjoint)
   double pad;
   double cd[20];
-  float cl[20];
+  float cl[16];
 };
 static_assert(sizeof(InstDev) % 16 == 0, "descriptor size");
-static_assert(kNumCoef <= 20, "coefficient slots");
+static_assert(kNumCoef <= 16 && kNumCoef64 <= 20, "coefficient slots");
 
 // One tile of one instance: {instance, x0, y0, partial slot, masked}.
 // masked: the tile holds a solid node or a node with a solid neighbour along
