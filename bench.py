@@ -167,6 +167,16 @@ def measured_peaks():
         return 6800.0, "fallback"
 
 
+def reduction_launches(insts) -> int:
+    """Launches of the end-of-call reduction of float32 instances: two stages
+    where an instance has more than 512 tiles (96 nodes each, at most 32 wide),
+    else one."""
+    def tiles(inst):
+        tx = min(inst.nx, 32)
+        return -(-inst.nx // tx) * -(-inst.ny // (96 // tx))
+    return 2 if max(tiles(i) for i in insts) > 512 else 1
+
+
 def kernel_sources_sha256() -> str:
     import hashlib
     h = hashlib.sha256()
@@ -679,9 +689,7 @@ def run_ours(args):
                           "lbve_step(K), lbve_fields_many (every instance to pinned host, "
                           "one synchronisation)"},
         "flops": measured_flops(value),
-        # K steps and the two stages of the end-of-call reduction (one where every
-        # instance has at most 512 tiles of 96 nodes)
-        "gpu_launches": K + (2 if max(i.n_nodes for i in insts) > 512 * 96 else 1),
+        "gpu_launches": K + reduction_launches(insts),
         "clocks": clocks,
         "fp64_plain": {"value": value64, "unit": UNIT, "steps": K64, "ms_per_step": ms64 / K64,
                        "kernel_ms": kernel_ms64,
