@@ -32,8 +32,8 @@ static AdjArgs<R> cast_args(const AdjArgsRaw& a) {
 }
 
 template <typename R, typename K>
-static void launch(K kernel, int blocks, int threads, const InstDev* d, const AdjArgs<R>& A,
-                   cudaStream_t st) {
+static void launch(K kernel, int blocks, int threads, bool overlap, const InstDev* d,
+                   const AdjArgs<R>& A, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(blocks);
   cfg.blockDim = dim3(threads);
@@ -42,26 +42,35 @@ static void launch(K kernel, int blocks, int threads, const InstDev* d, const Ad
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &attr;
-  // float64 passes of more than half an SM each would put early CTAs beside running
-  // ones on the same float64 pipe (128^2, 50 steps: 5.0 ms without, 6.0 with)
-  cfg.numAttrs = sizeof(R) == 4 || 2 * blocks <= kNumSMs ? 1 : 0;
+  cfg.numAttrs = overlap ? 1 : 0;
   cudaLaunchKernelEx(&cfg, kernel, d, A);
 }
 
 // OPEN: the node passes' variant with an open channel's inlet and outlet
 // columns (one-sided x-differences there in every mode, the column pass's
 // completion in the step modes).
+// Whether a pass launches with the programmatic dependency, i.e. starts while the
+// one before it ends.  Float32: always.  Float64: CTAs that arrive early share an
+// SM's float64 pipe and registers with running ones once they are more than the
+// idle SMs hold, so each pass decides by its own CTAs: at most a third of the SMs
+// of 256 threads; for the local pass, whose CTAs fill half an SM's registers, at
+// most 0.4 per SM.  50 steps in ms, all passes plain / all early / by this rule:
+// 64^2 3.53 / 3.20 / 3.25, 88^2 3.72 / 3.54 / 3.53, 92^2 3.88 / 4.00 / 3.70 (from
+// here on the local pass is plain), 96^2 3.70 / 4.18 / 3.49, 112^2 4.25 / 4.04 /
+// 4.03, 120^2 4.29 / 4.88 / 4.29 (from here on all are), 128^2 4.26 / 5.13 / 4.26.
 template <typename R, int MODE, bool OPEN, bool PUSH>
 static void run_pass(int pass, const InstDev* d, const AdjArgs<R>& A, int blocks, cudaStream_t st) {
+  const int local = blocks * (256 / kAdjLocalThreads);
+  const bool early = sizeof(R) == 4 || 3 * blocks <= kNumSMs;
+  const bool early_local = sizeof(R) == 4 || 5 * local <= 2 * kNumSMs;
   switch (pass) {
-    case 0: launch(adj_moments<R, MODE, OPEN>, blocks, 256, d, A, st); break;
+    case 0: launch(adj_moments<R, MODE, OPEN>, blocks, 256, early, d, A, st); break;
     case 1:
-      launch(adj_local<R, MODE, OPEN, PUSH>, blocks * (256 / kAdjLocalThreads), kAdjLocalThreads, d,
-             A, st);
+      launch(adj_local<R, MODE, OPEN, PUSH>, local, kAdjLocalThreads, early_local, d, A, st);
       break;
-    case 2: launch(adj_gather<R, MODE, OPEN, PUSH>, blocks, 256, d, A, st); break;
-    case 4: launch(adj_column<R, MODE>, blocks, 256, d, A, st); break;
-    default: launch(adj_pull<R>, blocks, 256, d, A, st); break;
+    case 2: launch(adj_gather<R, MODE, OPEN, PUSH>, blocks, 256, early, d, A, st); break;
+    case 4: launch(adj_column<R, MODE>, blocks, 256, early, d, A, st); break;
+    default: launch(adj_pull<R>, blocks, 256, early, d, A, st); break;
   }
 }
 
