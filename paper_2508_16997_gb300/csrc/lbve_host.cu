@@ -1615,6 +1615,8 @@ extern "C" int lbve_autotune(const lbve_params* p, int32_t n, void* d_workspace,
 // ---------------------------------------------------------------------------
 namespace {
 
+constexpr int64_t kAdjPiece = 64;  // forward steps whose descriptors go up together
+
 struct AdjPlan {
   int64_t T, s, nck;             // steps, checkpoint interval, checkpoints
   size_t state_bytes;            // one stored state: 41 planes
@@ -1625,16 +1627,17 @@ struct AdjPlan {
   int nwall, nmtiles;
   size_t off_scratch, off_walls, off_wrec, off_widx, off_mtiles;
   size_t off_cols;  // open channels: the column tasks of the instance (2 ny)
-  // Descriptors, one per kind of step, uploaded once: each names the state it
-  // reads and the one it writes.  (Uploaded before each step, with a device copy
-  // of the history, they took 15 % of a reversed step on a 512^2 grid.)
-  size_t desc_init() const { return 0; }                      // staged fields -> checkpoint 0
-  size_t desc_roll(int64_t m) const { return 1 + m; }         // segment state m % 2 -> (m + 1) % 2
-  size_t desc_leave(int64_t j) const { return 3 + j; }        // checkpoint j -> segment 0 (or j + 1)
-  size_t desc_enter(int64_t j) const { return 3 + nck + j; }  // last rolling state -> checkpoint j
-  size_t desc_seg(int64_t m) const { return 3 + 2 * nck + m; }        // segment state m -> m + 1
-  size_t desc_rev(int64_t m) const { return 3 + 2 * nck + s + m; }    // reverse of segment state m
-  size_t ndesc() const { return 3 + 2 * nck + 2 * s + 2; }
+  // Descriptors, each naming the state that a step reads and the one it writes:
+  // those of a segment's steps are uploaded once, those of the forward sweep in
+  // pieces of kAdjPiece, so that the table does not grow with the stored states.
+  // (Uploaded before each step, with a device copy of the history, they took 15 %
+  // of a reversed step on a 512^2 grid.)
+  size_t desc_init() const { return 0; }  // staged fields -> checkpoint 0
+  size_t desc_rev() const { return 1; }   // the reverse passes, of any state
+  size_t desc_seg(int64_t m) const { return 2 + m; }  // segment state m -> m + 1
+  size_t desc_piece() const { return 2 + (s - 1); }   // the forward sweep's
+  int64_t nforward() const { return (nck - 1) * s; }  // its steps
+  size_t ndesc() const { return desc_piece() + std::min(kAdjPiece, nforward()); }
 };
 
 // The square-root checkpoint interval: ceil(sqrt(T)).
@@ -1669,10 +1672,11 @@ AdjPlan make_adj_plan(const lbve_params& p, const InstPlan& q, int64_t T, int nw
   a.off_fields = take(sizeof(double) * 6 * q.stride);
   a.off_stage = take(sizeof(double) * 6 * q.stride);
   a.off_ck = take(a.state_bytes * a.nck);
-  a.off_seg = take(a.state_bytes * (a.s + 1));
+  a.off_seg = a.s > 1 ? take(a.state_bytes * a.s) : off;  // interval 1: all in checkpoints
   a.off_lam[0] = take(a.state_bytes);
   a.off_lam[1] = take(a.state_bytes);
-  a.off_pulled = take(36 * plane);
+  // without a mask or open columns the first two passes write lambda_t themselves
+  a.off_pulled = nwall > 0 || nmtiles > 0 || p.open_x ? take(36 * plane) : off;
   a.off_G = take(6 * plane);
   a.off_dir = take(3 * plane);
   a.off_mh = take(8 * plane);
@@ -1857,32 +1861,28 @@ extern "C" int lbve_adjoint_step_ex(lbve_handle* h, int32_t inst, const double* 
   // the completion)
   auto ckp = [&](int64_t j) { return ck + j * a.state_bytes; };
   auto segp = [&](int64_t m) { return seg + m * a.state_bytes; };
-  std::vector<InstDev> descs(a.ndesc(), D);
-  auto put_desc = [&](size_t at, char* from, char* to) {
-    InstDev& E = descs[at];
+  auto step_desc = [&](char* from, char* to) -> InstDev {
+    InstDev E = D;
     E.pop[0] = masked ? scratch : from;
     E.pop[1] = to;
     E.hist = hist_of(from);
     E.hist_out = hist_of(to);
+    return E;
   };
-  {
-    InstDev& E = descs[a.desc_init()];
-    E.pop[0] = stage;
-    E.pop[1] = ck;
-    E.hist = E.hist_out = hist_of(ck);
-  }
-  for (int64_t m = 0; m < 2; ++m)
-    if (a.s > 1) put_desc(a.desc_roll(m), segp(m), segp(1 - m));
-  for (int64_t j = 0; j < a.nck; ++j) {
-    put_desc(a.desc_leave(j), ckp(j), a.s > 1 ? segp(0) : ckp(std::min(j + 1, a.nck - 1)));
-    if (a.s > 1) put_desc(a.desc_enter(j), segp((a.s - 2) % 2), ckp(j));
-  }
-  for (int64_t m = 0; m + 1 < a.s; ++m) put_desc(a.desc_seg(m), segp(m), segp(m + 1));
+  // (a pageable source is staged before the call returns)
+  auto put_descs = [&](size_t at, const std::vector<InstDev>& v) -> cudaError_t {
+    return v.empty() ? cudaSuccess
+                     : cudaMemcpyAsync(d_desc + at, v.data(), sizeof(InstDev) * v.size(),
+                                       cudaMemcpyHostToDevice, st);
+  };
+  std::vector<InstDev> descs(2, D);
+  descs[a.desc_init()].pop[0] = stage;
+  descs[a.desc_init()].pop[1] = ck;
+  descs[a.desc_init()].hist = descs[a.desc_init()].hist_out = hist_of(ck);
   // the reverse passes take sizes, coefficients and flags from theirs; the state
   // comes with their arguments
-  for (int64_t m = 0; m < a.s; ++m) put_desc(a.desc_rev(m), segp(m), segp(m));
-  e = cudaMemcpyAsync(d_desc, descs.data(), sizeof(InstDev) * descs.size(), cudaMemcpyHostToDevice,
-                      st);
+  for (int64_t m = 0; m + 1 < a.s; ++m) descs.push_back(step_desc(segp(m), segp(m + 1)));
+  e = put_descs(0, descs);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_fail(e, "adjoint set-up");
 
@@ -1904,12 +1904,22 @@ extern "C" int lbve_adjoint_step_ex(lbve_handle* h, int32_t inst, const double* 
   // ---- forward sweep: X_0 from the initial fields, checkpoints every s steps ----
   if (!launch_tiles(a.desc_init(), kModeInit, kFinal))
     return cuda_fail(cudaGetLastError(), "adjoint init step");
-  for (int64_t j = 1; j < a.nck; ++j) {
-    // X_{j s} from X_{(j-1) s}: s steps through two rolling buffers of the segment area
-    int rc = fwd(a.desc_leave(j - 1), ckp(j - 1));
-    for (int64_t m = 1; m < a.s && !rc; ++m)
-      rc = fwd(m == a.s - 1 ? a.desc_enter(j) : a.desc_roll((m - 1) % 2), segp((m - 1) % 2));
-    if (rc) return rc;
+  // step i of the sweep leads from X_i to X_{i+1}; between two checkpoints the
+  // states alternate between the first two of the segment area
+  auto swept = [&](int64_t i) -> char* {
+    const int64_t m = i % a.s;
+    return m == 0 ? ckp(i / a.s) : segp((m - 1) % 2);
+  };
+  for (int64_t i0 = 0; i0 < a.nforward(); i0 += kAdjPiece) {
+    const int64_t i1 = std::min(i0 + kAdjPiece, a.nforward());
+    descs.clear();
+    for (int64_t i = i0; i < i1; ++i) descs.push_back(step_desc(swept(i), swept(i + 1)));
+    if ((e = put_descs(a.desc_piece(), descs)) != cudaSuccess)
+      return cuda_fail(e, "adjoint descriptors");
+    for (int64_t i = i0; i < i1; ++i) {
+      const int rc = fwd(a.desc_piece() + (i - i0), swept(i));
+      if (rc) return rc;
+    }
   }
 
   // ---- reverse sweep ----
@@ -1972,7 +1982,7 @@ extern "C" int lbve_adjoint_step_ex(lbve_handle* h, int32_t inst, const double* 
     }
     for (int64_t m = m1 - 1; m >= m0; --m) {
       char* X = a.s > 1 ? segp(m - m0) : ckp(j);
-      const size_t at = a.desc_rev(m - m0);
+      const size_t at = a.desc_rev();
       A.X = X;
       A.lam_cur = lam[li ^ 1];
       int mode;
