@@ -12,7 +12,7 @@
 //   u = (j + F/2)/rho, moments       -> lambda of the completed populations
 //   Zou-He and CNEBB completions     -> lambda of pulled populations, own wall slots, u_b
 //   pull streaming                   -> reverse pull (a gather from x + e_i)
-// Three passes per step, each one thread per node:
+// Two or three passes per step, each one thread per node:
 //   adj_local   collision/source/CNEBB reverse at the node; writes lambda of the
 //               conformation pulls, the gradient adjoints and the direct
 //               adjoints of rho and u; writes lambda_t's history part
@@ -163,7 +163,7 @@ __device__ __forceinline__ R bouzidi(const InstDev& D, const R* X, const WallDev
 
 // Open channels: the inlet (x = 0) and outlet (x = nx - 1) nodes' completed
 // populations come from the neighbouring column x_f = 1 or nx - 2, as the
-// forward column pass builds them: the neighbour's pull, Zou-He and CNEBB on
+// forward edge pass builds them: the neighbour's pull, Zou-He and CNEBB on
 // wall rows, its rho, u and phi, then
 //   inlet:  f = f_f + f^eq(rho_f, u_in) - f^eq(rho_f, u_f),
 //           g = g_f + g^eq(A_in, u_in) - g^eq(phi_f, u_f);
@@ -317,7 +317,7 @@ __device__ __forceinline__ void adj_hydro_node(const InstDev& D, const AdjArgs<R
     pull9<R>(A.X, S, y * nx, rm, rp, x, xm, xp, d);
     if (!py && (y == 0 || y == ny - 1)) zou_he<R>(d, Fx, Fy, y == 0);
     if (A.widx && A.widx[k] >= 0) {
-      // the wall pass: interpolated bounce-back of the wall links
+      // the edge pass: interpolated bounce-back of the wall links
       const WallDev& W = A.walls[A.widx[k]];
 #pragma unroll
       for (int i = 1; i < 9; ++i)
@@ -460,7 +460,7 @@ __device__ __forceinline__ void cnebb_T(const R d[9], R pa, R pb, R pc, R delta,
 }
 
 // CNEBB at a fluid node next to the mask (Sec. 3.3), unknown set U = umask,
-// as the wall pass does it: pm[i] (i in U) is the node's own post-collision
+// as the edge pass does it: pm[i] (i in U) is the node's own post-collision
 // slot opposite i.
 template <typename R>
 __device__ __forceinline__ void cnebb_mask(R g[9], const R pm[9], R delta, R ubx, R uby,
@@ -1008,7 +1008,7 @@ __global__ void adj_gather(const InstDev* __restrict__ Dp, AdjArgs<R> A) {
   A.dF[n + k] += (double)lFy;
 }
 
-// Pass 2b (open channels, after the gather): reverse of the column pass.
+// Pass 2b (open channels, after the gather): reverse of the edge pass's columns.
 // One thread per open-column node (side, y).  The gather and the local pass
 // left there lambda of the node's completed populations; they go back to the
 // neighbour x_f's pulled populations (the unknown slots of a wall row carry

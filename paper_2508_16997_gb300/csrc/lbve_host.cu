@@ -527,10 +527,10 @@ void update_geometry_hash(lbve_handle* h, int i) {
 // whose halo region (all TX x TY slots -- a ragged tile fills the slots past
 // the edge with the wrapped nodes -- one column left and right, hy rows above
 // and below), grown by one node, holds a solid node or a node of an open
-// column.  Then no plain tile reads a slot the wall pass writes (solid nodes'
+// column.  Then no plain tile reads a slot the edge pass writes (solid nodes'
 // slots, wall nodes' rest slots) or an open column's node, so plain tiles
-// need not wait for the wall and column passes.  Rebuilds the list's
-// masked-tile table and uploads both tables.
+// need not wait for the edge pass.  Rebuilds the list's masked-tile table and
+// uploads both tables.
 int flag_tiles(lbve_handle* h, int i) {
   const lbve_params& p = h->p[i];
   const InstPlan& q = h->plan.inst[i];
@@ -960,7 +960,7 @@ static int init_geometry(lbve_handle* h, int32_t n, const int32_t* ids, const in
   }
   // pageable sources: the copies are staged before the calls return.  The
   // descriptors go up as one array when the list covers much of the handle,
-  // else one by one (a single instance of a large batch moves 400 bytes)
+  // else one by one (a single instance of a large batch moves one)
   cudaError_t e = cudaMemcpyAsync(h->d_geo, geo.data(), sizeof(int32_t) * geo.size(),
                                   cudaMemcpyHostToDevice, h->stream);
   if ((size_t)n * 8 >= (size_t)h->n) {
@@ -1622,7 +1622,7 @@ struct AdjPlan {
   size_t state_bytes;            // one stored state: 41 planes
   size_t off_desc, off_tiles, off_partials, off_fields, off_stage, off_ck, off_seg, off_lam[2],
       off_pulled, off_G, off_dir, off_mh, off_M, off_zero, total;
-  // solid masks: the raw-state scratch the wall pass completes, the wall
+  // solid masks: the raw-state scratch the edge pass completes, the wall
   // records and final-step records, each node's record, the masked tiles
   int nwall, nmtiles;
   size_t off_scratch, off_walls, off_wrec, off_widx, off_mtiles;
@@ -1798,7 +1798,7 @@ extern "C" int lbve_adjoint_step_ex(lbve_handle* h, int32_t inst, const double* 
   std::vector<WallDev> wcopy;
   std::vector<int32_t> widx;
   if (open) {
-    // the column pass of instance 0 (the inlet profile is the instance's)
+    // the edge pass's column nodes of instance 0 (the inlet profile is the instance's)
     std::vector<ColTask> cols(2 * size_t(p.ny));
     for (int side = 0; side < 2; ++side)
       for (int y = 0; y < p.ny; ++y) cols[side * p.ny + y] = ColTask{0, y, side, 0};
@@ -1856,7 +1856,7 @@ extern "C" int lbve_adjoint_step_ex(lbve_handle* h, int32_t inst, const double* 
                           st);
   }
   if (e != cudaSuccess) return cuda_fail(e, "adjoint initial-field upload");
-  // the descriptors of every step; with a mask the wall pass completes a scratch
+  // the descriptors of every step; with a mask the edge pass completes a scratch
   // copy of the state read, so stored states stay raw (the reverse passes redo
   // the completion)
   auto ckp = [&](int64_t j) { return ck + j * a.state_bytes; };

@@ -214,7 +214,7 @@ struct AdjArgsRaw {
              // no reverse pull
 };
 // pass: 0 moments, 1 local reverse, 2 gather, 3 reverse pull, 4 reverse of an
-// open channel's column pass (n_nodes = 2 ny: one thread per open-column
+// open channel's columns (n_nodes = 2 ny: one thread per open-column
 // node); mode: kAdjStep, kAdjFields, kAdjInit (lbve_adjoint.cuh).
 int launch_adjoint(int prec, int mode, int pass, const InstDev* d_desc, const AdjArgsRaw& a,
                    int n_nodes, void* stream);

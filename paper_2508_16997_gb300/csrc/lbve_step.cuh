@@ -1040,7 +1040,7 @@ struct MinBlocks {
 };
 
 // Open channels: nodes of the inlet (x = 0) and outlet (x = nx - 1) columns
-// take their completed populations from the column pass's colbuf during a
+// take their completed populations from the edge pass's colbuf during a
 // step (the pull would miss the populations entering from outside).
 __device__ __forceinline__ bool open_column(const InstDev& D, int gx) {
   return D.open_x && (gx == 0 || gx == D.nx - 1);
