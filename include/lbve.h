@@ -413,7 +413,7 @@ int lbve_adjoint_step(lbve_handle* h, int32_t inst, const double* init_fields,
  *                  the gradient with respect to the wall geometry; needs a
  *                  solid mask.
  * At least one of d_dL_dfields and dL_ddrag must be given.  The forward
- * states are recomputed with the wall pass; the reverse passes differentiate
+ * states are recomputed with the edge pass; the reverse passes differentiate
  * the interpolated bounce-back, CNEBB at the mask and the one-sided
  * gradients next to solid nodes.
  * Errors: as lbve_adjoint_step(); LBVE_ERR_GEOMETRY for drag or q gradients
